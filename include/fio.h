@@ -28,12 +28,18 @@
  * head and a TF32 tail and a product is summed as head*head + head*tail + tail*head (three MMAs
  * per step, FP32 accumulation; the dropped tail*tail term is ~2^-22 relative); same factors and
  * vectors as FIO_PTF32.  With fewer than 8 right-hand sides the tensor-core precisions fall back
- * to the FP32 CUDA-core kernels.  FIO_PDF takes complex128 vectors and applies a double-float copy
+ * to the FP32 CUDA-core kernels.  The large stages of FIO_P64 and FIO_P32 run on the tensor cores in
+ * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below their row's and column's largest,
+ * digit products summed exactly, each output rounded once -- at least as close to the exact product
+ * as the CUDA-core sums (columns with infinities, NaN or extreme exponents are summed plainly).
+ * FIO_PDF takes complex128 vectors and applies a double-float copy
  * of the factors (each FP64 entry as an unevaluated sum of two floats, 48-bit significand) with
  * compensated (twice-working-precision) accumulation on the FP32 CUDA cores: FP64-class results
  * (~1e-14 relative per stage) at the FP32 pipes' rate, for the outer residual of iterative
  * refinement (GB300's FP64 rate is a small fraction of its FP32 rate); it adds two conversion
- * launches per apply and is not accepted by fio_apply_inv_noalloc.  The vector dtype
+ * launches per apply and is not accepted by fio_apply_inv_noalloc.  Where every stage of the operator
+ * runs in fixed point (operators above 4096 unknowns with both copies), FIO_PDF runs as FIO_P64: more
+ * accurate than double-float, and faster.  The vector dtype
  * must match the precision (C128 with P64 and PDF, C64 with the others); other pairs return FIO_EINVAL.
  *
  * STREAMS AND SCRATCH.  Calls are asynchronous on `stream` (a cudaStream_t; NULL = the legacy
@@ -204,7 +210,8 @@ int fio_solve(fio_op op, const void* u, void* f, int64_t ld, int b, int dtype,
  * product on the butterfly stages (Gauss's 3M form: the imaginary part's rounding error up to a
  * few times the four-product one; the in-place HIF stages keep four products), 17 (FP32) the
  * tiles of 9 with 16-column chunks, 18 (FP32) the tiles of 11 without their register cap (three
- * CTAs per SM instead of four); with a tensor-core
+ * CTAs per SM instead of four), 50 (FP64 and FP32) the fixed-point tensor-core kernel on the stages
+ * that have its copy (also the built-in choice where it is the faster one); with a tensor-core
  * precision and b >= 8: 0 the single-buffer tcgen05 kernel, 20 / 21 / 22 its warp-specialised
  * ring variant with 2 / 3 / 4 chunk stages, 30 the persistent tcgen05 kernel whose factor tiles
  * arrive by TMA (work units of as many 128-row tiles as tensor memory holds, deepest ring), 31
@@ -215,15 +222,15 @@ int fio_solve(fio_op op, const void* u, void* f, int64_t ld, int b, int dtype,
  * stages.  Stages whose rows are not 16-byte aligned (an odd width in a hand-packed buffer) and
  * odd b keep variant 0 or the FP32 CUDA cores.
  * Every variant sums each output's terms in the same order, except 8 (tree reductions), 12 and
- * 31 (the in-place stages' slices) and 14..16 (three products), so results for b >= 5 do not
- * depend on the choice otherwise.  choices (may be NULL when cap == 0) receives
+ * 31 (the in-place stages' slices), 14..16 (three products) and 50 (exact sums), so results for
+ * b >= 5 do not depend on the choice otherwise.  choices (may be NULL when cap == 0) receives
  * the variant per stage launch in stage order, forward before adjoint (the root: forward
  * only); *nchoices (may be NULL) their number.  Synchronises `stream`; must not run
  * concurrently with other calls on the operator. */
 int fio_autotune(fio_op op, int b, int precision, void* stream, int* choices, int cap, int* nchoices);
 
 /* Pin the kernel variant of every stage launch of (precision, the bucket of b) to `variant`
- * (0 = the built-in choice): 1..18 as for fio_autotune on the CUDA cores (8 only for b <= 4,
+ * (0 = the built-in choice): 1..18 and 50 as for fio_autotune on the CUDA cores (50 not for FIO_PDF; 8 only for b <= 4,
  * 9..12, 17, 18 only for FIO_P32, 13 not for FIO_PDF, 14..16 only for FIO_P64 and FIO_PDF); with a tensor-core precision and b >= 8, 0 (single-buffer kernel),
  * 20, 21, 22 (the warp-specialised ring kernel with 2, 3, 4 chunk stages), 30..33 (the
  * TMA-fed persistent kernel, as for fio_autotune) or 40 (FP32 CUDA cores); a variant that does not apply to a stage
@@ -267,7 +274,8 @@ int fio_apply_profiled(fio_op op, int which, const void* x, void* y, int64_t ld,
  * critical loop where the implicit device synchronisation of cudaMalloc/cudaFree is not
  * acceptable.  fio_apply_inv may grow the operator's scratch pool on a larger b; this variant
  * never allocates and never frees: its scratch is a static device array of
- * FIO_NOALLOC_SCRATCH_BYTES that every device loading libfio holds until the process exits.
+ * FIO_NOALLOC_SCRATCH_BYTES that every device loading libfio holds until the process exits (and
+ * one of half that size for the fixed-point stages).
  *
  * Same arguments, result and errors as fio_apply_inv, plus: FIO_EINVAL when the call needs more
  * scratch than the static array holds (3 work vectors of max_len x b elements, max_len the

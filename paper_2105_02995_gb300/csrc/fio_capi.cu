@@ -381,6 +381,11 @@ extern "C" int fio_upload_factors(const void* packed, size_t nbytes, unsigned ma
       return urc;
     }
   }
+  const int fxrc = fx_build(op, meta, mdims, s);
+  if (fxrc != FIO_OK) {
+    fio_release(op);
+    return fxrc;
+  }
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
     fio_release(op);
     return FIO_ECUDA;
@@ -397,6 +402,7 @@ extern "C" int fio_release(fio_op op) {
   if (op->arena_df) cudaFree(op->arena_df);
   if (op->meta) cudaFree(op->meta);
   if (op->units) cudaFree(op->units);
+  if (op->fx) cudaFree(op->fx);
   if (op->arena_tc) cudaFree(op->arena_tc);
   if (op->scratch) cudaFree(op->scratch);
   fio_solver_free(op);
@@ -412,7 +418,7 @@ extern "C" int fio_query(fio_op op, int* d, int64_t* n, int64_t* N, size_t* devi
   if (N) *N = op->N;
   if (device_bytes)
     *device_bytes = op->arena_bytes + op->arena32_bytes + op->arena_tc_bytes + op->arena_df_bytes + op->meta_bytes +
-                    op->units_bytes + op->scratch_bytes + op->solver_bytes;
+                    op->units_bytes + op->fx_bytes + op->scratch_bytes + op->solver_bytes;
   return FIO_OK;
 }
 
@@ -433,10 +439,11 @@ extern "C" const char* fio_strerror(int status) {
 // ---------------------------------------------------------------------------------------------
 // scratch pool: 5 work arrays of max(max_len, N) x b complex elements each
 // ---------------------------------------------------------------------------------------------
-int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs) {
+int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void** fxbuf, size_t* fxbytes) {
   const size_t per = (size_t)op->max_len * (size_t)b * elem;
   const size_t per_al = (per + 255) & ~(size_t)255;
-  const size_t need = 5 * per_al;
+  const size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
+  const size_t need = 5 * per_al + fxneed;
   if (need > op->scratch_bytes) {
     if (op->scratch) {
       if (cudaStreamSynchronize(s) != cudaSuccess) return FIO_ECUDA;
@@ -451,6 +458,8 @@ int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs) {
     op->scratch_bytes = need;
   }
   for (int k = 0; k < 5; ++k) bufs[k] = (uint8_t*)op->scratch + k * per_al;
+  if (fxbuf) *fxbuf = fxneed ? (uint8_t*)op->scratch + 5 * per_al : nullptr;
+  if (fxbytes) *fxbytes = fxneed;
   return FIO_OK;
 }
 
@@ -971,6 +980,56 @@ StageArgs<V> stage_args(const Stage& st, bool adj, const V* x, long long xrs, lo
   return a;
 }
 
+// ---- fixed-point tensor-core kernel (fio_fx.cuh): variant 50, and the built-in choice of the
+// stages it takes.  Its scratch is set for the duration of one public call (FxScratch); without
+// one the CUDA-core kernels serve.
+constexpr int kFxVariant = 50;
+thread_local void* g_fx_scratch = nullptr;
+thread_local size_t g_fx_bytes = 0;
+struct FxScratch {
+  void* prev;
+  size_t prev_bytes;
+  FxScratch(void* p, size_t n) : prev(g_fx_scratch), prev_bytes(g_fx_bytes) {
+    g_fx_scratch = p;
+    g_fx_bytes = n;
+  }
+  ~FxScratch() {
+    g_fx_scratch = prev;
+    g_fx_bytes = prev_bytes;
+  }
+};
+// whether the kernel can run this launch, and (pinned false) whether it is the built-in choice
+template <typename V>
+bool fx_rule(const Stage& st, bool adj, int b, bool pinned) {
+  constexpr bool W = std::is_same<V, double2>::value;
+  if (std::is_same<V, dfc>::value || !g_fx_scratch || (!W && g_tc_mode != 0)) return false;
+  return st.fx_ok[W ? 0 : 1] && (pinned || fx_takes(st, adj, W, b));
+}
+// device address of the timeout flag (the kernel is in another translation unit), cached per device
+int* timeout_flag() {
+  static std::mutex mu;
+  static std::map<int, int*> cache;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  int*& p = cache[dev];
+  void* q = nullptr;
+  if (!p && cudaGetSymbolAddress(&q, g_tc_timeout) == cudaSuccess) p = (int*)q;
+  if (!p) cudaGetLastError();
+  return p;
+}
+template <typename V>
+bool launch_fx(const Stage& st, bool adj, const V* x, long long xrs, long long xcs, V* y, long long yrs, long long ycs,
+               int b, cudaStream_t s, bool pinned) {
+  if (!fx_rule<V>(st, adj, b, pinned)) return false;
+  int* flag = timeout_flag();
+  return flag && fx_launch(st, adj, std::is_same<V, double2>::value, x, xrs, xcs, y, yrs, ycs, b, g_fx_scratch, g_fx_bytes,
+                           flag, s);
+}
+
 template <typename V>
 void launch_stage(const Stage& st, bool adj, const V* x, long long xrs, long long xcs, V* y,
                   long long yrs, long long ycs, int b, cudaStream_t s) {
@@ -985,6 +1044,7 @@ void launch_stage(const Stage& st, bool adj, const V* x, long long xrs, long lon
   }
   const StageArgs<V> a = stage_args<V>(st, adj, x, xrs, xcs, y, yrs, ycs, b);
   int var = st.var[type_index<V>()][adj ? 1 : 0][rhs_bucket(b)];
+  if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, x, xrs, xcs, y, yrs, ycs, b, s, var == kFxVariant)) return;
   if (st.kind == 1) var = four_product_of(var);  // in-place stages keep four products
   if (adj) launch_stage_dir<V, true>(a, s, var);
   else launch_stage_dir<V, false>(a, s, var);
@@ -1162,9 +1222,11 @@ void apply_core(fio_op op, Which w, const V* x, V* y, int64_t ld, int b, V* A, V
 
 template <typename V>
 int apply_t(fio_op op, Which w, const void* xv, void* yv, int64_t ld, int b, cudaStream_t s) {
-  void* bufs[5];
-  int rc = fio_scratch(op, b, sizeof(V), s, bufs);
+  void *bufs[5], *fxb;
+  size_t fxn;
+  int rc = fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn);
   if (rc) return rc;
+  FxScratch fxs(fxb, fxn);
   apply_core<V>(op, w, (const V*)xv, (V*)yv, ld, b, (V*)bufs[0], (V*)bufs[1], (V*)bufs[2], s);
   return finish(s);
 }
@@ -1184,8 +1246,20 @@ int apply_df(fio_op op, Which w, const void* xv, void* yv, int64_t ld, int b, cu
   return finish(s);
 }
 
+// Whether FIO_PDF runs as FIO_P64: when every stage has the fixed-point kernel's FP64 copy, that
+// kernel is both faster than double-float arithmetic on the FP32 pipes (2D n = 256, K-dot at b = 16:
+// 3.4 ms against 15) and more accurate (exact sums of 62-bit operands against 48-bit ones).  A
+// double-float variant pinned by fio_set_variant keeps the double-float kernels.
+bool df_as_fp64(fio_op op, int b) {
+  if (!fx_all_wide(op)) return false;
+  const int k = rhs_bucket(b);
+  for (const auto& st : op->st)
+    if (st.var[2][0][k] || st.var[2][1][k]) return false;
+  return true;
+}
+
 int apply_prec(fio_op op, Which w, const void* x, void* y, int64_t ld, int b, int prec, cudaStream_t s) {
-  if (prec == FIO_P64) return apply_t<double2>(op, w, x, y, ld, b, s);
+  if (prec == FIO_P64 || (prec == FIO_PDF && df_as_fp64(op, b))) return apply_t<double2>(op, w, x, y, ld, b, s);
   if (prec == FIO_PDF) return apply_df(op, w, x, y, ld, b, s);
   TcMode m(tc_mode_of(prec));
   return apply_t<float2>(op, w, x, y, ld, b, s);
@@ -1247,8 +1321,8 @@ extern "C" int fio_apply_inv_host(fio_op op, const void* u_host, void* f_host, i
   if (b == 0) return FIO_OK;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t es = dtype == FIO_C128 ? 16 : 8;
-  void* bufs[5];
-  int rc = fio_scratch(op, b, es, s, bufs);
+  void *bufs[5], *fxb;  // asked for with its scratch, so that the apply below does not grow it again
+  int rc = fio_scratch(op, b, es, s, bufs, &fxb);
   if (rc) return rc;
   void *U = bufs[3], *F = bufs[4];
   const size_t w = (size_t)op->N * es;
@@ -1367,9 +1441,11 @@ constexpr int kTcCand[9] = {0,  20, 21, 22, kTmaVariant, kTmaSplitVariant, kTmaB
 // per (stage, direction) in stage order, forward before adjoint
 template <typename V>
 int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch) {
-  void* bufs[5];
-  int rc = fio_scratch(op, b, sizeof(V), s, bufs);
+  void *bufs[5], *fxb;
+  size_t fxn;
+  int rc = fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn);
   if (rc) return rc;
+  FxScratch fxs(fxb, fxn);
   const size_t bytes = (size_t)op->max_len * b * sizeof(V);
   V* X = (V*)bufs[0];
   V* Y = (V*)bufs[1];
@@ -1395,17 +1471,18 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
       if (st.nblk > 0) {
         const StageArgs<V> a = stage_args<V>(st, adj, X, b, 1, Y, b, 1, b);
         float tbest = -1.f;
-        const int ncand = tc ? 9 : kNCand;
+        const int ncand = tc ? 9 : kNCand + 1;
         for (int k = 0; k < ncand; ++k) {
-          const int var = tc ? kTcCand[k] : kCand[bucket][k];
-          if (var <= 0 && !tc) break;
+          const int var = tc ? kTcCand[k] : (k == kNCand ? kFxVariant : kCand[bucket][k]);
+          if (var <= 0 && !tc) continue;
+          if (var == kFxVariant && !fx_rule<V>(st, adj, b, true)) continue;
           float t;
           if (st.kind == 1) {
             // in-place stages: the whole stage (compute and copy-back, or split compute and
             // reduction), so that the split variant is weighed with its reduction
             t = time_launch(
                 [&] {
-                  if (!tc && (!variant_applies<V>(a, var) || is_3m_variant(var))) return false;
+                  if (!tc && var != kFxVariant && (!variant_applies<V>(a, var) || is_3m_variant(var))) return false;
                   st.var[ti][dir][bucket] = (int8_t)var;
                   inplace_stage<V>(st, adj, X, Y, b, s, (V*)bufs[2], op->max_len);
                   return true;
@@ -1423,6 +1500,8 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
           } else if (tc) {
             t = time_launch([&] { return launch_tc(st, adj, (const float2*)X, b, 1, (float2*)Y, b, 1, b, s, var); },
                             s, e0, e1);
+          } else if (var == kFxVariant) {
+            t = time_launch([&] { return launch_fx<V>(st, adj, X, b, 1, Y, b, 1, b, s, true); }, s, e0, e1);
           } else if (adj) {
             t = time_launch([&] { return launch_variant<V, true>(a, s, var); }, s, e0, e1);
           } else {
@@ -1437,7 +1516,7 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
             best = var;
           }
         }
-        if (rc == FIO_OK && tc && fio_tc_timeout_reset() != 0) rc = FIO_ETIMEOUT;
+        if (rc == FIO_OK && (tc || best == kFxVariant) && fio_tc_timeout_reset() != 0) rc = FIO_ETIMEOUT;
       }
       st.var[ti][dir][bucket] = (int8_t)best;
       if (choices && n < cap) choices[n] = best;
@@ -1464,7 +1543,9 @@ extern "C" int fio_set_variant(fio_op op, int b, int precision, int variant) {
     ti = 2 + mode;
   } else {
     ti = precision == FIO_P64 ? 0 : (precision == FIO_PDF ? 2 : 1);
-    if (variant < 0 || variant > kMaxCudaCoreVariant || (variant == 8 && b > kVecMaxRhs) ||
+    if (variant == kFxVariant && ti != 2) {
+      // the fixed-point kernel where it takes the stage (also the built-in choice there)
+    } else if (variant < 0 || variant > kMaxCudaCoreVariant || (variant == 8 && b > kVecMaxRhs) ||
         (is_fp32_tile_variant(variant) && ti != 1) || (variant == kSmallVariant && ti == 2) ||
         (is_3m_variant(variant) && ti == 1))
       return FIO_EINVAL;
@@ -1492,7 +1573,7 @@ extern "C" int fio_autotune(fio_op op, int b, int precision, void* stream, int* 
   }
   g_tune_flush = flush;
   int rc;
-  if (precision == FIO_P64) {
+  if (precision == FIO_P64 || (precision == FIO_PDF && df_as_fp64(op, b))) {
     rc = tune_type<double2>(op, b, s, choices, cap, nchoices);
   } else if (precision == FIO_PDF) {
     rc = tune_type<dfc>(op, b, s, choices, cap, nchoices);
@@ -1542,6 +1623,9 @@ __global__ void k_to_c64(const double2* a, float2* b, long long n) {
 void convert_in(const double2* a, float2* b, long long n, cudaStream_t s) {
   k_to_c64<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, b, n);
 }
+void convert_in(const double2* a, double2* b, long long n, cudaStream_t s) {
+  cudaMemcpyAsync(b, a, (size_t)n * sizeof(double2), cudaMemcpyDeviceToDevice, s);
+}
 void convert_in(const double2* a, dfc* b, long long n, cudaStream_t s) {
   k_split_df<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, b, (size_t)n);
 }
@@ -1558,6 +1642,10 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
             cudaMalloc(&W64, len * sizeof(double2)) == cudaSuccess && cudaMalloc(&A, len * sizeof(V)) == cudaSuccess &&
             cudaMalloc(&B, len * sizeof(V)) == cudaSuccess && cudaMalloc(&W, len * sizeof(V)) == cudaSuccess &&
             cudaMalloc(&acc, 2 * sizeof(double)) == cudaSuccess;
+  const size_t fxn = std::max(fx_scratch_bytes(op, b, sizeof(double2)), fx_scratch_bytes(op, b, sizeof(float2)));
+  void* fxb = nullptr;
+  if (ok && fxn) ok = cudaMalloc(&fxb, fxn) == cudaSuccess;
+  FxScratch fxs(fxb, fxn);
   int rc = ok ? FIO_OK : FIO_ENOMEM;
   int k = 0;
   auto record = [&](const double2* ref, const V* val, long long n) {
@@ -1617,6 +1705,7 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
   cudaFree(B);
   cudaFree(W);
   cudaFree(acc);
+  if (fxb) cudaFree(fxb);
   cudaGetLastError();
   if (nerr) *nerr = k;
   if (rc == FIO_OK && fio_tc_timeout_reset() > 0) rc = FIO_ETIMEOUT;
@@ -1634,6 +1723,7 @@ extern "C" int fio_stage_errors(fio_op op, int which, const void* x, int64_t ld,
   if (which >= 2 && op->n_root == 0) return FIO_ENOTSUP;
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaGetLastError() != cudaSuccess) return FIO_ECUDA;
+  if (precision == FIO_PDF && df_as_fp64(op, b)) return stage_errors_t<double2>(op, which, x, ld, b, s, errs, cap, nerr);
   if (precision == FIO_PDF) return stage_errors_t<dfc>(op, which, x, ld, b, s, errs, cap, nerr);
   TcMode m(tc_mode_of(precision));
   return stage_errors_t<float2>(op, which, x, ld, b, s, errs, cap, nerr);
@@ -1647,13 +1737,18 @@ extern "C" int fio_stage_errors(fio_op op, int which, const void* x, int64_t ld,
 // exits.  Host code must not use the array's name as a device address: its address on the
 // current device comes from cudaGetSymbolAddress, taken once per device on the first call there.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[FIO_NOALLOC_SCRATCH_BYTES];
+// the fixed-point kernel's scratch beside it: a gathered vector, at most 1.5 times a work vector but
+// for blocks of a few columns (a stage that does not fit runs on the CUDA cores)
+constexpr size_t kNoallocFxBytes = FIO_NOALLOC_SCRATCH_BYTES / 2;
+static __device__ __align__(256) unsigned char g_noalloc_fx[kNoallocFxBytes];
 
 namespace {
 constexpr int kNoallocMaxDevices = 64;
 void* g_noalloc_addr[kNoallocMaxDevices];
+void* g_noalloc_fx_addr[kNoallocMaxDevices];
 std::mutex g_noalloc_mu;
 
-int noalloc_scratch(void** out) {
+int noalloc_scratch(void** out, void** fx) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
@@ -1667,9 +1762,16 @@ int noalloc_scratch(void** out) {
       cudaGetLastError();
       return FIO_ECUDA;
     }
+    void* q = nullptr;
+    if (cudaGetSymbolAddress(&q, g_noalloc_fx) != cudaSuccess || !q) {
+      cudaGetLastError();
+      return FIO_ECUDA;
+    }
     g_noalloc_addr[dev] = p;
+    g_noalloc_fx_addr[dev] = q;
   }
   *out = g_noalloc_addr[dev];
+  *fx = g_noalloc_fx_addr[dev];
   return FIO_OK;
 }
 
@@ -1692,9 +1794,10 @@ extern "C" int fio_apply_inv_noalloc(fio_op op, const void* u, void* f, int64_t 
   const size_t es = precision == FIO_P64 ? sizeof(double2) : sizeof(float2);
   const size_t per = (((size_t)op->max_len * (size_t)b * es) + 255) & ~(size_t)255;
   if (per > FIO_NOALLOC_SCRATCH_BYTES / 3) return FIO_EINVAL;  // does not fit the static scratch
-  void* base = nullptr;
-  rc = noalloc_scratch(&base);
+  void *base = nullptr, *fxb = nullptr;
+  rc = noalloc_scratch(&base, &fxb);
   if (rc) return rc;
+  FxScratch fxs(fxb, kNoallocFxBytes);
   if (cudaGetLastError() != cudaSuccess) return FIO_ECUDA;
   uint8_t* p = (uint8_t*)base;
   cudaStream_t s = (cudaStream_t)stream;

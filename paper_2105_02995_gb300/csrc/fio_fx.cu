@@ -1,0 +1,290 @@
+// fio_fx.cu -- host side of the fixed-point tensor-core stage kernel (fio_fx.cuh): which stages it
+// takes, their digit copies and work units at upload, and its launches.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <map>
+#include <mutex>
+#include <type_traits>
+#include <vector>
+
+#include "fio.h"
+#include "fio_fx.cuh"
+#include "fio_internal.h"
+
+using namespace fio;
+
+namespace {
+
+// Stages the kernel may take.  In operators of at most kSmallOp unknowns only those with at least
+// kMinUnits 128-row tiles: their small and in-place stages keep the CUDA-core sums, which every tile
+// shape reproduces bit for bit.  Above, FP64 takes every stage (a CUDA-core FP64 tile of a 28-row
+// block takes 55 us whatever the number of blocks; this kernel 8 us), FP32 those with kMinUnits
+// tiles whose blocks have more than kSmallDim rows or columns.
+constexpr int64_t kSmallOp = 4096;
+constexpr int kMinUnits = 96;
+constexpr int kSmallDim = 32;
+
+inline size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+template <typename R, bool ADJ>
+void pack(const Stage& st, const FxUnit* units, uint8_t* A, cudaStream_t s) {
+  using V = typename fx::Cfg<R>::V;
+  const V* M = (const V*)(std::is_same<R, double>::value ? (const void*)st.M64 : (const void*)st.M32);
+  k_fx_pack<R, ADJ><<<st.n_fx_units[ADJ], 256, 0, s>>>(units, M, ADJ ? st.in : st.out, ADJ ? st.out : st.in, st.fx_exp[ADJ],
+                                                       (int)st.R, (int)st.C, A);
+}
+
+// dynamic shared memory opt-in, once per device and kernel
+bool opt_in(const void* f, int bytes) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, int> granted;
+  std::lock_guard<std::mutex> lock(mu);
+  int& cap = granted[std::make_pair(dev, f)];
+  if (bytes <= cap) return true;
+  if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cap = bytes;
+  return true;
+}
+
+int sm_count() {
+  static std::mutex mu;
+  static std::map<int, int> known;
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::lock_guard<std::mutex> lock(mu);
+  int& k = known[dev];
+  if (k == 0) k = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 1;
+  return k;
+}
+
+template <typename R, bool ADJ, int BT>
+bool launch(FxArgs a, uint8_t* X, int* ej, cudaStream_t s) {
+  a.nrt = (a.b + BT - 1) / BT;
+  constexpr int fixed = fx::smem_fixed<R, BT>(), raw = fx::raw_bytes<BT>();
+  a.nraw = std::min(fx::kMaxRaw, (227 * 1024 - 512 - fixed) / raw);  // 512: the static barriers
+  const int need = fixed + a.nraw * raw;
+  const long long total = (long long)a.nunits * a.nrt;
+  if (total > 0x7fffffffLL || a.nrt > 65535) return false;
+  if (!opt_in((const void*)k_stage_fx<R, ADJ, BT>, need)) return false;
+  k_fx_gather<R, ADJ, BT><<<dim3((unsigned)a.nblk, (unsigned)a.nrt), 256, 0, s>>>(a, X, ej);
+  k_stage_fx<R, ADJ, BT><<<(unsigned)std::min<long long>(total, sm_count()), fx::kThreads, need, s>>>(a);
+  return true;
+}
+
+template <typename R, bool ADJ>
+bool launch_b(const FxArgs& a, uint8_t* X, int* ej, cudaStream_t s) {
+  if (a.b <= 8) return launch<R, ADJ, 8>(a, X, ej, s);
+  if constexpr (std::is_same<R, float>::value)
+    if (a.b > 16) return launch<R, ADJ, 32>(a, X, ej, s);
+  return launch<R, ADJ, 16>(a, X, ej, s);
+}
+
+}  // namespace
+
+int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>& mdims, cudaStream_t s) {
+  const bool want[2] = {(op->mask & FIO_MASK_P64) != 0, (op->mask & FIO_MASK_P32) != 0 && op->arena32};
+  if (!want[0] && !want[1]) return FIO_OK;
+  struct Plan {
+    int stage;
+    bool want[2];
+    size_t units[2], exps, xofs[2], digits[2][2];  // offsets: entries, entries, entries, bytes
+  };
+  std::vector<Plan> plans;
+  std::vector<FxUnit> units;
+  std::vector<int2> xofs;
+  size_t nexp = 0, dbytes = 0;
+  for (size_t si = 0; si < op->st.size(); ++si) {
+    Stage& st = op->st[si];
+    int2 n = make_int2(0, 0);
+    bool ok = st.nblk > 0;
+    for (uint32_t b = 0; ok && b < st.nblk; ++b) {
+      const int2 d = meta[mdims[si] + b];
+      ok = d.x > 0 && d.y > 0;
+      st.nnz = (b ? st.nnz : 0) + (long long)d.x * d.y;
+      n.x += (d.x + 127) / 128;
+      n.y += (d.y + 127) / 128;
+    }
+    const bool few = std::min(n.x, n.y) < kMinUnits;
+    Plan p;
+    p.stage = (int)si;
+    p.want[0] = ok && want[0] && (op->N > kSmallOp || !few);
+    p.want[1] = ok && want[1] && !few && std::max(st.maxcols[0], st.maxcols[1]) > kSmallDim;
+    if (!p.want[0] && !p.want[1]) continue;
+    p.exps = nexp;
+    nexp += (size_t)st.nblk * (st.R + st.C);
+    long long cols[2] = {0, 0};
+    size_t bytes[2][2];
+    const size_t u0 = units.size(), x0 = xofs.size();
+    for (int dir = 0; dir < 2; ++dir) {
+      p.units[dir] = units.size();
+      p.xofs[dir] = xofs.size();
+      long long xo[2] = {0, 0};
+      for (uint32_t b = 0; b < st.nblk; ++b) {
+        const int2 d = meta[mdims[si] + b];
+        const int rows = dir ? d.y : d.x, c = dir ? d.x : d.y;
+        for (int r0 = 0; r0 < rows; r0 += 128) units.push_back(FxUnit{(int)b, r0, rows, c, 0, 0, (int)xo[0], (int)xo[1]});
+        xofs.push_back(make_int2((int)xo[0], (int)xo[1]));
+        xo[0] += (c + 7) / 8 * 8;
+        xo[1] += (c + 15) / 16 * 16;
+      }
+      for (int t = 0; t < 2; ++t) cols[t] = std::max(cols[t], xo[t]);
+      st.fx_cols[dir] = make_int2((int)xo[0], (int)xo[1]);
+      std::stable_sort(units.begin() + p.units[dir], units.end(), [](const FxUnit& x, const FxUnit& y) { return x.ncols > y.ncols; });
+      long long at[2] = {0, 0};  // 128-byte rows of the digit copies
+      for (size_t k = p.units[dir]; k < units.size(); ++k) {
+        FxUnit& u = units[k];
+        const int rp = std::min(128, (u.nrows - u.r0 + 31) & ~31);
+        u.a64 = (int)at[0];
+        u.a32 = (int)at[1];
+        at[0] += (long long)rp * ((u.ncols + 7) / 8);
+        at[1] += (long long)rp * ((u.ncols + 15) / 16);
+      }
+      ok = ok && std::max(at[0], at[1]) < 0x7fffffffLL && std::max(xo[0], xo[1]) < 0x7fffffffLL;
+      for (int t = 0; t < 2; ++t) bytes[t][dir] = (size_t)at[t] * 128;
+      st.n_fx_units[dir] = (int)(units.size() - p.units[dir]);
+      st.fx_steps[dir] = 0;
+      for (size_t k = p.units[dir]; k < units.size(); ++k) st.fx_steps[dir] += (units[k].ncols + 7) / 8;
+    }
+    if (!ok) {
+      units.resize(u0);
+      xofs.resize(x0);
+      continue;
+    }
+    for (int t = 0; t < 2; ++t)
+      for (int dir = 0; p.want[t] && dir < 2; ++dir) {
+        p.digits[t][dir] = dbytes;
+        dbytes += al256(bytes[t][dir]);
+      }
+    for (int t = 0; t < 2; ++t) op->fx_max_cols[t] = std::max(op->fx_max_cols[t], cols[t]);
+    op->fx_max_blk = std::max(op->fx_max_blk, (long long)st.nblk);
+    plans.push_back(p);
+  }
+  if (plans.empty()) return FIO_OK;
+  const size_t oe = al256(units.size() * sizeof(FxUnit)), ox = oe + al256(nexp * sizeof(short)),
+               ob = ox + al256(xofs.size() * sizeof(int2)), od = ob + al256(plans.size() * sizeof(int));
+  if (cudaMalloc(&op->fx, od + dbytes) != cudaSuccess) {  // no room for the copies: the CUDA-core kernels serve
+    cudaGetLastError();
+    op->fx = nullptr;
+    op->fx_max_cols[0] = op->fx_max_cols[1] = 0;
+    return FIO_OK;
+  }
+  op->fx_bytes = od + dbytes;
+  uint8_t* p0 = (uint8_t*)op->fx;
+  int* bad = (int*)(p0 + ob);
+  if (cudaMemcpyAsync(p0, units.data(), units.size() * sizeof(FxUnit), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemcpyAsync(p0 + ox, xofs.data(), xofs.size() * sizeof(int2), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemsetAsync(p0 + oe, 0, ox - oe, s) != cudaSuccess || cudaMemsetAsync(bad, 0, od - ob, s) != cudaSuccess)
+    return FIO_ECUDA;
+  for (size_t k = 0; k < plans.size(); ++k) {
+    const Plan& p = plans[k];
+    Stage& st = op->st[p.stage];
+    short* re = (short*)(p0 + oe) + p.exps;
+    st.fx_exp[0] = re;
+    st.fx_exp[1] = re + (size_t)st.nblk * st.R;
+    k_fx_exps<<<st.nblk, 512, 0, s>>>(st.M64, st.in, st.out, st.dims, (int)st.R, (int)st.C, re, re + (size_t)st.nblk * st.R,
+                                      bad + k);
+    for (int dir = 0; dir < 2; ++dir) {
+      st.fx_units[dir] = (const FxUnit*)p0 + p.units[dir];
+      st.fx_xofs[dir] = (const int2*)(p0 + ox) + p.xofs[dir];
+      for (int t = 0; t < 2; ++t) st.fxA[t][dir] = p.want[t] ? p0 + od + p.digits[t][dir] : nullptr;
+    }
+    if (p.want[0]) {
+      pack<double, false>(st, st.fx_units[0], p0 + od + p.digits[0][0], s);
+      pack<double, true>(st, st.fx_units[1], p0 + od + p.digits[0][1], s);
+    }
+    if (p.want[1]) {
+      pack<float, false>(st, st.fx_units[0], p0 + od + p.digits[1][0], s);
+      pack<float, true>(st, st.fx_units[1], p0 + od + p.digits[1][1], s);
+    }
+  }
+  std::vector<int> hbad(plans.size(), 1);
+  if (cudaMemcpyAsync(hbad.data(), bad, plans.size() * sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return FIO_ECUDA;
+  for (size_t k = 0; k < plans.size(); ++k)
+    for (int t = 0; t < 2; ++t) op->st[plans[k].stage].fx_ok[t] = plans[k].want[t] && !hbad[k];
+  return FIO_OK;
+}
+
+size_t fx_scratch_bytes(fio_op op, int b, size_t elem) {
+  const int t = elem == sizeof(double2) ? 0 : 1;
+  if (!op->fx || op->fx_max_cols[t] == 0) return 0;
+  return al256((size_t)op->fx_max_cols[t] * (size_t)b * elem) + al256((size_t)op->fx_max_blk * (size_t)b * sizeof(int));
+}
+
+// The built-in choice.  FP64 from b = 5 on: the CUDA-core kernels need 4 to 20 times as long on every
+// stage.  FP64 at b <= 4 (k_stage_vec streams the factor at 0.8 TFLOP/s forward, 1.1 adjoint) and FP32
+// by estimated time: K steps of the busiest SM at the measured time a step, against the CUDA-core rate
+// (31 TFLOP/s up to 16 right-hand sides, 42 above).  Measured on both sides of the line: blocks of
+// 415 x 250 at FP32 b = 32 0.34 ms against 0.60, of 58 x 58 0.035 against 0.030; FP64 b = 1 58 x 58
+// adjoint 0.0319 against 0.0290, 415 x 250 0.38 against 0.75.  FP32 also needs two tiles for every SM:
+// below, the few tiles' own latency decides and the smaller CUDA-core tiles fill the chip better.
+bool fx_takes(const Stage& st, bool adj, bool wide, int b) {
+  if (!st.fx_ok[wide ? 0 : 1]) return false;
+  const int sms = sm_count(), bt = wide ? (b <= 8 ? 8 : 16) : (b <= 8 ? 8 : b <= 16 ? 16 : 32);
+  const long long nrt = (b + bt - 1) / bt, units = st.n_fx_units[adj] * nrt;
+  // microseconds: K steps of the busiest SM, against the CUDA-core kernels' rate
+  const double step = wide ? (bt == 8 ? 0.55 : 0.80) : (bt == 8 ? 0.33 : bt == 16 ? 0.37 : 0.45);
+  const double waves = (double)((units + sms - 1) / sms) / ((double)units / sms);
+  const double fx = 4.0 + step * waves * (double)(st.fx_steps[adj] * nrt) / sms;
+  if (wide) return b > 4 || fx < 8e-6 * (double)st.nnz * b / (adj ? 1.1 : 0.8);
+  const int bp = b <= 16 ? 16 : (b + 31) / 32 * 32;
+  return b > 8 && units >= 2LL * sms && fx < 8e-6 * (double)st.nnz * bp / (b <= 16 ? 31.0 : 42.0);
+}
+
+bool fx_all_wide(fio_op op) {
+  for (const Stage& st : op->st)
+    if (st.nblk && !st.fx_ok[0]) return false;
+  return op->fx != nullptr;
+}
+
+bool fx_launch(const Stage& st, bool adj, bool wide, const void* x, long long xrs, long long xcs, void* y, long long yrs,
+               long long ycs, int b, void* scratch, size_t scratch_bytes, int* timeout, cudaStream_t s) {
+  const int dir = adj ? 1 : 0;
+  const size_t elem = wide ? sizeof(double2) : sizeof(float2);
+  const long long cols = wide ? st.fx_cols[dir].x : st.fx_cols[dir].y;
+  const size_t xb = al256((size_t)cols * (size_t)b * elem);
+  if (!scratch || xb + (size_t)st.nblk * (size_t)b * sizeof(int) > scratch_bytes) return false;
+  FxArgs a;
+  a.units = st.fx_units[dir];
+  a.nunits = st.n_fx_units[dir];
+  a.nrt = 1;
+  a.A = st.fxA[wide ? 0 : 1][dir];
+  a.X = (const uint8_t*)scratch;
+  a.ej = (const int*)((uint8_t*)scratch + xb);
+  a.rexp = st.fx_exp[dir];
+  a.rowidx = adj ? st.in : st.out;
+  a.colidx = adj ? st.out : st.in;
+  a.lrow = adj ? (int)st.C : (int)st.R;
+  a.lcol = adj ? (int)st.R : (int)st.C;
+  a.dims = st.dims;
+  a.xofs = st.fx_xofs[dir];
+  a.xcols = cols;
+  a.nblk = (int)st.nblk;
+  a.R = (int)st.R;
+  a.C = (int)st.C;
+  a.M = wide ? (const void*)st.M64 : (const void*)st.M32;
+  a.x = x;
+  a.xrs = xrs;
+  a.xcs = xcs;
+  a.y = y;
+  a.yrs = yrs;
+  a.ycs = ycs;
+  a.b = b;
+  a.nraw = 0;
+  a.timeout = timeout;
+  uint8_t* X = (uint8_t*)scratch;
+  int* ej = (int*)(X + xb);
+  if (wide) return adj ? launch_b<double, true>(a, X, ej, s) : launch_b<double, false>(a, X, ej, s);
+  return adj ? launch_b<float, true>(a, X, ej, s) : launch_b<float, false>(a, X, ej, s);
+}

@@ -14,6 +14,13 @@ namespace fio {
 
 struct dfc;  // double-float complex (fio_kernels.cuh)
 
+// work unit of the fixed-point kernel (fio_fx.cuh): one 128-row tile of a block in one direction
+struct FxUnit {
+  int blk, r0, nrows, ncols;  // block, first row of the tile, valid rows and columns of the block
+  int a64, a32;               // where its digits start in the FP64 / FP32 copy (128-byte rows)
+  int x64, x32;               // columns before the block in the gathered vector
+};
+
 struct Stage {
   uint32_t kind, nblk, R, C;
   int64_t in_len, out_len;
@@ -54,6 +61,18 @@ struct Stage {
   // first 128-row tile, tiles, 0), largest first
   const int4* units[2][3] = {};
   int nunits[2][3] = {};
+  // fixed-point kernel per [forward, adjoint]: scale exponents of the product's rows, work units,
+  // column offsets of the blocks in the gathered vector and its columns, and the digit copies of
+  // the factor per [FP64, FP32][direction]; fx_ok: the copies exist and every exponent is in range
+  bool fx_ok[2] = {};
+  const short* fx_exp[2] = {};
+  const FxUnit* fx_units[2] = {};
+  int n_fx_units[2] = {};
+  const int2* fx_xofs[2] = {};
+  int2 fx_cols[2] = {};
+  long long fx_steps[2] = {0, 0};  // K steps (8 columns) of all units
+  long long nnz = 0;               // block entries, padding excluded
+  const uint8_t* fxA[2][2] = {};
 };
 
 }  // namespace fio
@@ -79,6 +98,10 @@ struct fio_op_s {
   size_t meta_bytes = 0;
   void* units = nullptr;          // work-unit lists of the TMA kernel (every stage)
   size_t units_bytes = 0;
+  void* fx = nullptr;             // digit copies, scale exponents and work units of the fixed-point kernel
+  size_t fx_bytes = 0;
+  long long fx_max_cols[2] = {0, 0};  // most columns of a gathered vector (FP64, FP32 chunking)
+  long long fx_max_blk = 0;           // most blocks of a stage it takes
   void* solver = nullptr;         // solver work arrays (fio_solve.cu)
   size_t solver_bytes = 0;
 };
@@ -86,8 +109,20 @@ struct fio_op_s {
 // precisions whose stage products may run on the tensor cores (complex64 vectors)
 inline bool is_tc_precision(int p) { return p == FIO_PTF32 || p == FIO_PBF16 || p == FIO_PTF32X3; }
 
-// scratch work arrays (5 of max_len x b elements of `elem` bytes); grows with a stream sync
-int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs);
+// fixed-point tensor-core stage kernel (fio_fx.cu): its copies at upload (synchronises s); the
+// scratch that its launches need for b right-hand sides of `elem` bytes; whether it takes a stage
+// launch; the launch (false: not taken, nothing launched; *timeout is set by a bounded wait that gives up)
+int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>& mdims, cudaStream_t s);
+size_t fx_scratch_bytes(fio_op op, int b, size_t elem);
+bool fx_takes(const fio::Stage& st, bool adj, bool wide, int b);
+bool fx_all_wide(fio_op op);  // every stage of the operator has an FP64 digit copy
+bool fx_launch(const fio::Stage& st, bool adj, bool wide, const void* x, long long xrs, long long xcs, void* y,
+               long long yrs, long long ycs, int b, void* scratch, size_t scratch_bytes, int* timeout, cudaStream_t s);
+
+// scratch work arrays (5 of max_len x b elements of `elem` bytes); grows with a stream sync;
+// fxbuf (may be null) receives the fixed-point kernel's scratch behind them, fxbytes its size
+int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void** fxbuf = nullptr,
+                size_t* fxbytes = nullptr);
 // which: 0 K-dot, 1 K-dot*, 2 G-dot, 3 G-dot K-dot*; x, y column-major with leading dimension ld
 int fio_apply_internal(fio_op op, int which, const void* x, void* y, int64_t ld, int b, int prec,
                        cudaStream_t s);

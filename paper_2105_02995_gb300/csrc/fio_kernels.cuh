@@ -921,7 +921,7 @@ __global__ void k_row_to_col(const V* W, V* Y, long long ld, long long N, int b)
   }
 }
 
-__global__ void k_cast_c128_c64(const double2* a, float2* b, size_t n) {
+static __global__ void k_cast_c128_c64(const double2* a, float2* b, size_t n) {
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) b[t] = make_float2((float)a[t].x, (float)a[t].y);
 }
@@ -931,18 +931,18 @@ __device__ __forceinline__ dfc split_df(double2 v) {
   const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
   return dfc{rh, ih, __double2float_rn(v.x - (double)rh), __double2float_rn(v.y - (double)ih)};
 }
-__global__ void k_split_df(const double2* a, dfc* b, size_t n) {
+static __global__ void k_split_df(const double2* a, dfc* b, size_t n) {
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) b[t] = split_df(a[t]);
 }
 // N x b column-major complex128 (leading dimension ld) -> double-float (leading dimension N), and back
-__global__ void k_c128_to_df(const double2* x, long long ld, dfc* y, long long N, int b) {
+static __global__ void k_c128_to_df(const double2* x, long long ld, dfc* y, long long N, int b) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const long long j = t / N, i = t - j * N;
   y[t] = split_df(x[j * ld + i]);
 }
-__global__ void k_df_to_c128(const dfc* y, long long N, double2* x, long long ld, int b) {
+static __global__ void k_df_to_c128(const dfc* y, long long N, double2* x, long long ld, int b) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const long long j = t / N, i = t - j * N;

@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(192) k_stage_tc_ring(TcArgs a) {
 
 // Self-test of the bounded wait: every CTA waits on an mbarrier that nothing arrives at, with a
 // limit of limit_ns; the wait must give up, record the timeout and return.
-__global__ void k_wait_selftest(uint64_t limit_ns, int* gave_up) {
+static __global__ void k_wait_selftest(uint64_t limit_ns, int* gave_up) {
   using namespace tc;
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x == 0) mbar_init(&bar, 1);
@@ -625,7 +625,7 @@ __global__ void k_wait_selftest(uint64_t limit_ns, int* gave_up) {
 }
 
 // block-wise transpose of the complex64 copy: out block (C x R) = in block (R x C)^T
-__global__ void k_transpose_blocks(const float2* in, float2* out, int nblk, int R, int C) {
+static __global__ void k_transpose_blocks(const float2* in, float2* out, int nblk, int R, int C) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long per = (long long)R * C;
   if (t >= per * nblk) return;
@@ -635,7 +635,7 @@ __global__ void k_transpose_blocks(const float2* in, float2* out, int nblk, int 
 }
 
 // bf16 copy with row stride ld (>= cols, padding zero): out[b][r][0..ld) from in[b][r][0..cols)
-__global__ void k_to_bf16(const float2* in, __nv_bfloat162* out, int nblk, int rows, int cols, int ld) {
+static __global__ void k_to_bf16(const float2* in, __nv_bfloat162* out, int nblk, int rows, int cols, int ld) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long per = (long long)rows * ld;
   if (t >= per * nblk) return;
