@@ -381,7 +381,8 @@ extern "C" int fio_upload_factors(const void* packed, size_t nbytes, unsigned ma
       return urc;
     }
   }
-  const int fxrc = fx_build(op, meta, mdims, s);
+  int fxrc = fft_build(op, s);
+  if (fxrc == FIO_OK) fxrc = fx_build(op, meta, mdims, s);
   if (fxrc != FIO_OK) {
     fio_release(op);
     return fxrc;
@@ -403,6 +404,7 @@ extern "C" int fio_release(fio_op op) {
   if (op->meta) cudaFree(op->meta);
   if (op->units) cudaFree(op->units);
   if (op->fx) cudaFree(op->fx);
+  if (op->fft_tw) cudaFree(op->fft_tw);
   if (op->arena_tc) cudaFree(op->arena_tc);
   if (op->scratch) cudaFree(op->scratch);
   fio_solver_free(op);
@@ -418,7 +420,7 @@ extern "C" int fio_query(fio_op op, int* d, int64_t* n, int64_t* N, size_t* devi
   if (N) *N = op->N;
   if (device_bytes)
     *device_bytes = op->arena_bytes + op->arena32_bytes + op->arena_tc_bytes + op->arena_df_bytes + op->meta_bytes +
-                    op->units_bytes + op->fx_bytes + op->scratch_bytes + op->solver_bytes;
+                    op->units_bytes + op->fx_bytes + op->fft_bytes + op->scratch_bytes + op->solver_bytes;
   return FIO_OK;
 }
 

@@ -8,12 +8,17 @@
 // exp(-+2 pi i x.xi) = (-1)^(k_1+..+k_d) exp(-+2 pi i k.j/n): F is the standard DFT of the
 // sign-modulated input scaled by n^{-d}, F^{-1} the sign-modulated standard inverse DFT.
 //
-// Kernel: k_fft_pass, a batch of power-of-two transforms of length L <= 2048 in shared memory,
-// 2048 / L transforms per CTA (one right-hand side per grid row).  Element e of transform t is
-// read at t*xt + e*xe and written at t*yt + e*ye of the right-hand side's vector, so one kernel
-// serves the contiguous and the strided axes; the copies walk whichever index is contiguous in
-// memory.  In shared memory: elements loaded to bit-reversed positions, then log2 L in-place
-// radix-2 butterfly stages (twiddles from a per-CTA table of exp(s 2 pi i t/L), t < L/2).
+// Kernel: k_fft_pass, a batch of power-of-two transforms of length L <= 2048, 2048 / L transforms per
+// CTA of 256 threads (one right-hand side per grid row).  Element e of transform t is read at
+// t*xt + e*xe and written at t*yt + e*ye of the right-hand side's vector, so one kernel serves the
+// contiguous and the strided axes; the threads walk whichever index is contiguous in memory.
+// Stockham's autosort form with eight values per thread in registers: one stage of radix 2 or 4
+// when log2 L is not a multiple of three, then stages of radix 8; the first stage reads and the last
+// one writes global memory, between them the values go through shared memory (L = 256: two
+// exchanges; a radix-2 form in shared memory needs a barrier and a round trip for each of its eight
+// stages, and took 74 us for the two passes of 32 transforms of 256 x 256 in FP32 against 29 us: now bound
+// by the latency of its loads and exchanges, at 2.3 TB/s through L2).
+// Twiddles exp(2 pi i k / 2048) come from a table made at upload.
 // Optional per-element factors: the (-1)^k sign modulation on the input (F) or on the output
 // (F^{-1}), the four-step twiddle exp(s 2 pi i t e / N) on the output, and a scale.
 // Plans: 2D n x n = transforms along i1, then along i2; 1D N <= 2048 = one pass; 1D N > 2048 =
@@ -39,7 +44,7 @@ struct FftPass {
   int T;               // transforms per right-hand side
   long long xt, xe;    // input offset of element e of transform t: t*xt + e*xe
   long long yt, ye;    // output offset
-  int sign;            // +1: exp(+2 pi i ...) (inverse DFT), -1: forward
+  const void* tw;      // exp(2 pi i k / 2048), k < 2048, in the vectors' precision
   int twN;             // > 0: multiply output (t, e) by exp(sign 2 pi i (t e mod twN) / twN)
   int mod_in, mod_out; // (-1)^(grid coordinate sum) of the input / output linear index
   int n, logn, d;      // grid (for the modulation)
@@ -58,92 +63,177 @@ template <> struct Cplx<double> {
   static __device__ __forceinline__ void sincospi_(double a, double* s, double* c) { sincospi(a, s, c); }
 };
 
-__device__ __forceinline__ bool odd_coord_sum(long long k, const FftPass& p) {
-  if (p.d == 1) return (k & 1) != 0;
-  return (((k & (p.n - 1)) + (k >> p.logn)) & 1) != 0;
+// (offsets within one right-hand side's vector fit an int: N <= 2^22)
+__device__ __forceinline__ bool odd_coord_sum(int k, const FftPass& p) {
+  return ((p.d == 1 ? k : k ^ (k >> p.logn)) & 1) != 0;
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kFftThreads) k_fft_pass(FftPass p) {
+template <typename V> __device__ __forceinline__ V cadd(V a, V b) { a.x += b.x; a.y += b.y; return a; }
+template <typename V> __device__ __forceinline__ V csub(V a, V b) { a.x -= b.x; a.y -= b.y; return a; }
+template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
+  V r;
+  r.x = a.x * b.x - a.y * b.y;
+  r.y = a.x * b.y + a.y * b.x;
+  return r;
+}
+// a times exp(SIGN pi i / 2)
+template <int SIGN, typename V> __device__ __forceinline__ V times_i(V a) {
+  V r;
+  r.x = SIGN > 0 ? -a.y : a.y;
+  r.y = SIGN > 0 ? a.x : -a.x;
+  return r;
+}
+template <int SIGN, typename V> __device__ __forceinline__ void dft2(V& a, V& b) {
+  const V t = b;
+  b = csub(a, t);
+  a = cadd(a, t);
+}
+// in place, results in natural order
+template <int SIGN, typename V> __device__ __forceinline__ void dft4(V& a, V& b, V& c, V& d) {
+  const V s0 = cadd(a, c), s1 = csub(a, c), s2 = cadd(b, d), s3 = times_i<SIGN>(csub(b, d));
+  a = cadd(s0, s2);
+  b = cadd(s1, s3);
+  c = csub(s0, s2);
+  d = csub(s1, s3);
+}
+template <int SIGN, typename V> __device__ __forceinline__ void dft8(V (&v)[8]) {
+  V e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+  dft4<SIGN>(e0, e1, e2, e3);
+  dft4<SIGN>(o0, o1, o2, o3);
+  // o1 exp(SIGN pi i / 4), o2 exp(SIGN pi i / 2), o3 exp(SIGN 3 pi i / 4)
+  using S = decltype(o1.x);
+  const S h = (S)0.70710678118654752440;
+  const V q1 = times_i<SIGN>(o1), q3 = times_i<SIGN>(o3);
+  V w1 = cadd(o1, q1), w3 = csub(q3, o3);
+  w1.x *= h;
+  w1.y *= h;
+  w3.x *= h;
+  w3.y *= h;
+  const V w2 = times_i<SIGN>(o2);
+  v[0] = cadd(e0, o0);
+  v[4] = csub(e0, o0);
+  v[1] = cadd(e1, w1);
+  v[5] = csub(e1, w1);
+  v[2] = cadd(e2, w2);
+  v[6] = csub(e2, w2);
+  v[3] = cadd(e3, w3);
+  v[7] = csub(e3, w3);
+}
+
+// where element e of transform tl lies in shared memory: strides of 8 elements, and neighbouring
+// transforms of the strided axes, are spread over the banks
+constexpr int kFftPad = 2;
+constexpr int kFftShared = kFftElems + kFftElems / 16 + kFftPad * (kFftElems / 16);
+__device__ __forceinline__ int place(int tl, int e, int L) {
+  return tl * (L + (L >> 4) + (L >= 16 ? kFftPad : 0)) + e + (e >> 4);
+}
+
+// The stage of radix RX after stages of product Ns, for this thread's 8 / RX butterflies: butterfly
+// (transform tl, index j < L / RX) takes elements j + r L / RX, turned by exp(2 pi i r (j mod Ns) / (Ns RX)),
+// and leaves element (j / Ns) Ns RX + j mod Ns + r Ns.
+template <typename R, int SIGN, int RX>
+__device__ __forceinline__ void fft_stage(const FftPass& p, typename Cplx<R>::T* s, const typename Cplx<R>::T* x,
+                                          typename Cplx<R>::T* y, int t0, int Ns, bool e_fast, bool oe_fast) {
   using C = Cplx<R>;
   using V = typename C::T;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* s = reinterpret_cast<V*>(smem_raw);         // kFftElems
-  V* tw = s + kFftElems;                        // L/2 twiddles
-  const int L = p.L, TT = kFftElems / L;
-  const int t0 = blockIdx.x * TT;
-  const int j = blockIdx.y;
-  const V* x = reinterpret_cast<const V*>(p.x) + (long long)j * p.ldx;
-  V* y = reinterpret_cast<V*>(p.y) + (long long)j * p.ldy;
-  const int tid = threadIdx.x;
-
-  for (int q = tid; q < L / 2; q += kFftThreads) {
-    R sn, cs;
-    C::sincospi_((R)(2 * q) / (R)L, &sn, &cs);  // exact argument: 2q/L with L a power of two
-    tw[q] = C::make(cs, (R)p.sign * sn);
-  }
-  // load: element (t, e) -> s[tl*L + bitrev(e)]; the contiguous index varies fastest
-  const bool e_fast = p.xe == 1 || p.xt != 1;
-  for (int i = tid; i < TT * L; i += kFftThreads) {
-    int tl, e;
-    if (e_fast) {
-      tl = i / L;
-      e = i - tl * L;
+  constexpr int NB = 8 / RX, LOGRX = RX == 8 ? 3 : RX == 4 ? 2 : 1;
+  const int L = p.L, logLR = p.logL - LOGRX, logTT = 11 - p.logL, logNs = __ffs(Ns) - 1;  // all powers of two
+  const bool first = Ns == 1, last = Ns * RX == L;
+  const V* tw = reinterpret_cast<const V*>(p.tw);
+  const int xt = (int)p.xt, xe = (int)p.xe, yt = (int)p.yt, ye = (int)p.ye;
+  V v[NB][RX];
+  int tl[NB], j[NB];
+  // which of (transform, index) runs along the threads: as global memory wants it at the two ends
+  const bool fast = last ? oe_fast : e_fast;
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    const int i = threadIdx.x + kFftThreads * k;
+    tl[k] = fast ? i >> logLR : i & ((1 << logTT) - 1);
+    j[k] = fast ? i & ((1 << logLR) - 1) : i >> logTT;
+    if (first) {
+      const int at = (t0 + tl[k]) * xt + j[k] * xe, step = xe << logLR;
+      const bool on = t0 + tl[k] < p.T;
+#pragma unroll
+      for (int r = 0; r < RX; ++r) v[k][r] = on ? x[at + r * step] : C::make(0, 0);
+      if (p.mod_in) {
+#pragma unroll
+        for (int r = 0; r < RX; ++r)
+          if (odd_coord_sum(at + r * step, p)) v[k][r] = C::make(-v[k][r].x, -v[k][r].y);
+      }
     } else {
-      e = i / TT;
-      tl = i - e * TT;
+#pragma unroll
+      for (int r = 0; r < RX; ++r) v[k][r] = s[place(tl[k], j[k] + (r << logLR), L)];
     }
-    const int t = t0 + tl;
-    V v = C::make(0, 0);
-    if (t < p.T) {
-      const long long k = (long long)t * p.xt + (long long)e * p.xe;
-      v = x[k];
-      if (p.mod_in && odd_coord_sum(k, p)) v = C::make(-v.x, -v.y);
+    if (!first) {
+      const int q = (j[k] & (Ns - 1)) << (11 - logNs - LOGRX);
+#pragma unroll
+      for (int r = 1; r < RX; ++r) {
+        V w = tw[r * q];
+        if (SIGN < 0) w.y = -w.y;
+        v[k][r] = cmul(v[k][r], w);
+      }
     }
-    s[tl * L + (int)(__brev((unsigned)e) >> (32 - p.logL))] = v;
+    if constexpr (RX == 2) dft2<SIGN>(v[k][0], v[k][1]);
+    if constexpr (RX == 4) dft4<SIGN>(v[k][0], v[k][1], v[k][2], v[k][3]);
+    if constexpr (RX == 8) dft8<SIGN>(v[k]);
   }
-  __syncthreads();
-  // radix-2 butterflies, in place, spans 1, 2, 4, ..., L/2
-  for (int lh = 0; lh < p.logL; ++lh) {
-    const int half = 1 << lh;
-    for (int i = tid; i < TT * (L / 2); i += kFftThreads) {
-      const int tl = i / (L / 2), r = i - tl * (L / 2);
-      const int g = r >> lh, k = r & (half - 1);
-      const int a0 = tl * L + (g << (lh + 1)) + k, a1 = a0 + half;
-      const V w = tw[k << (p.logL - 1 - lh)];
-      const V u = s[a0], v = s[a1];
-      const V wv = C::make(w.x * v.x - w.y * v.y, w.x * v.y + w.y * v.x);
-      s[a0] = C::make(u.x + wv.x, u.y + wv.y);
-      s[a1] = C::make(u.x - wv.x, u.y - wv.y);
+  if (!first) __syncthreads();  // every value is read before any is replaced
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    const int e0 = ((j[k] >> logNs) << (logNs + LOGRX)) + (j[k] & (Ns - 1));
+    if (!last) {
+#pragma unroll
+      for (int r = 0; r < RX; ++r) s[place(tl[k], e0 + (r << logNs), L)] = v[k][r];
+      continue;
     }
-    __syncthreads();
-  }
-  // store: frequency e of transform t
-  const bool oe_fast = p.ye == 1 || p.yt != 1;
-  for (int i = tid; i < TT * L; i += kFftThreads) {
-    int tl, e;
-    if (oe_fast) {
-      tl = i / L;
-      e = i - tl * L;
-    } else {
-      e = i / TT;
-      tl = i - e * TT;
-    }
-    const int t = t0 + tl;
+    const int t = t0 + tl[k];
     if (t >= p.T) continue;
-    V v = s[tl * L + e];
-    if (p.twN > 0) {
-      const long long r = ((long long)t * e) % p.twN;
-      R sn, cs;
-      C::sincospi_((R)(2 * r) / (R)p.twN, &sn, &cs);
-      sn *= (R)p.sign;
-      v = C::make(cs * v.x - sn * v.y, cs * v.y + sn * v.x);
+    const int at = t * yt + e0 * ye, step = ye << logNs;
+#pragma unroll
+    for (int r = 0; r < RX; ++r) {
+      V u = v[k][r];
+      if (p.twN > 0) {
+        const int q = (t * (e0 + (r << logNs))) & (p.twN - 1);  // t e < N <= 2^22
+        R sn, cs;
+        C::sincospi_((R)(2 * q) / (R)p.twN, &sn, &cs);
+        u = cmul(u, C::make(cs, SIGN > 0 ? sn : -sn));
+      }
+      R sc = (R)p.scale;
+      if (p.mod_out && odd_coord_sum(at + r * step, p)) sc = -sc;
+      y[at + r * step] = C::make(sc * u.x, sc * u.y);
     }
-    const long long k = (long long)t * p.yt + (long long)e * p.ye;
-    R sc = (R)p.scale;
-    if (p.mod_out && odd_coord_sum(k, p)) sc = -sc;
-    y[k] = C::make(sc * v.x, sc * v.y);
   }
+  if (!last) __syncthreads();
+}
+
+template <typename R, int SIGN>
+__global__ void __launch_bounds__(kFftThreads) k_fft_pass(FftPass p) {
+  using V = typename Cplx<R>::T;
+  __shared__ V s[kFftShared];
+  const int t0 = blockIdx.x * (kFftElems / p.L);
+  const V* x = reinterpret_cast<const V*>(p.x) + (long long)blockIdx.y * p.ldx;
+  V* y = reinterpret_cast<V*>(p.y) + (long long)blockIdx.y * p.ldy;
+  const bool e_fast = p.xe == 1 || p.xt != 1, oe_fast = p.ye == 1 || p.yt != 1;
+  int Ns = 1;
+  const int rem = p.logL % 3;
+  if (rem == 1) {
+    fft_stage<R, SIGN, 2>(p, s, x, y, t0, Ns, e_fast, oe_fast);
+    Ns = 2;
+  } else if (rem == 2) {
+    fft_stage<R, SIGN, 4>(p, s, x, y, t0, Ns, e_fast, oe_fast);
+    Ns = 4;
+  }
+  for (; Ns < p.L; Ns *= 8) fft_stage<R, SIGN, 8>(p, s, x, y, t0, Ns, e_fast, oe_fast);
+}
+
+// exp(2 pi i k / 2048) in both precisions, the FP32 one rounded from FP64
+__global__ void k_fft_twiddles(double2* t64, float2* t32) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= kFftElems) return;
+  double sn, cs;
+  sincospi(2.0 * k / kFftElems, &sn, &cs);
+  t64[k] = make_double2(cs, sn);
+  t32[k] = make_float2((float)cs, (float)sn);
 }
 
 int ilog2(long long v) {
@@ -153,16 +243,11 @@ int ilog2(long long v) {
 }
 
 template <typename R>
-int run_pass(const FftPass& p, int b, cudaStream_t s) {
+int run_pass(const FftPass& p, bool inverse, int b, cudaStream_t s) {
   const int TT = kFftElems / p.L;
   dim3 grid((unsigned)((p.T + TT - 1) / TT), (unsigned)b);
-  const size_t smem = (size_t)(kFftElems + p.L / 2) * sizeof(typename Cplx<R>::T);
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_fft_pass<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return FIO_ECUDA;
-  }
-  k_fft_pass<R><<<grid, kFftThreads, smem, s>>>(p);
+  if (inverse) k_fft_pass<R, 1><<<grid, kFftThreads, 0, s>>>(p);
+  else k_fft_pass<R, -1><<<grid, kFftThreads, 0, s>>>(p);
   return FIO_OK;
 }
 
@@ -172,7 +257,7 @@ int apply_dft(fio_op op, bool inverse, const void* x, void* y, long long ld, int
   const int n = (int)op->n, d = op->d;
   const long long N = op->N;
   FftPass p{};
-  p.sign = inverse ? 1 : -1;
+  p.tw = sizeof(R) == 8 ? op->fft_tw : (const void*)((const double2*)op->fft_tw + kFftElems);
   p.n = n;
   p.logn = ilog2(n);
   p.d = d;
@@ -203,8 +288,8 @@ int apply_dft(fio_op op, bool inverse, const void* x, void* y, long long ld, int
     }
     a.logL = ilog2(a.L);
     c.logL = ilog2(c.L);
-    if ((rc = run_pass<R>(a, b, s))) return rc;
-    if ((rc = run_pass<R>(c, b, s))) return rc;
+    if ((rc = run_pass<R>(a, inverse, b, s))) return rc;
+    if ((rc = run_pass<R>(c, inverse, b, s))) return rc;
   } else {
     p.x = x;
     p.y = y;
@@ -218,7 +303,7 @@ int apply_dft(fio_op op, bool inverse, const void* x, void* y, long long ld, int
     p.mod_in = inverse ? 0 : 1;
     p.mod_out = inverse ? 1 : 0;
     p.scale = scale_last;
-    if ((rc = run_pass<R>(p, b, s))) return rc;
+    if ((rc = run_pass<R>(p, inverse, b, s))) return rc;
   }
   return cudaGetLastError() == cudaSuccess ? FIO_OK : FIO_ECUDA;
 }
@@ -246,6 +331,18 @@ int dft_entry(fio_op op, bool inverse, const void* x, void* y, int64_t ld, int b
 }
 
 }  // namespace
+
+int fft_build(fio_op op, cudaStream_t s) {
+  const size_t bytes = kFftElems * (sizeof(double2) + sizeof(float2));
+  if (cudaMalloc(&op->fft_tw, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    op->fft_tw = nullptr;
+    return FIO_ENOMEM;
+  }
+  op->fft_bytes = bytes;
+  k_fft_twiddles<<<kFftElems / 256, 256, 0, s>>>((double2*)op->fft_tw, (float2*)((double2*)op->fft_tw + kFftElems));
+  return FIO_OK;
+}
 
 extern "C" int fio_apply_F(fio_op op, const void* f, void* fhat, int64_t ld, int b, int dtype, int precision,
                            void* stream) {

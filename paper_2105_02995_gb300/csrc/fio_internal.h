@@ -102,6 +102,8 @@ struct fio_op_s {
   size_t fx_bytes = 0;
   long long fx_max_cols[2] = {0, 0};  // most columns of a gathered vector (FP64, FP32 chunking)
   long long fx_max_blk = 0;           // most blocks of a stage it takes
+  void* fft_tw = nullptr;         // DFT twiddles: exp(2 pi i k / 2048), 2048 double2 then 2048 float2
+  size_t fft_bytes = 0;
   void* solver = nullptr;         // solver work arrays (fio_solve.cu)
   size_t solver_bytes = 0;
 };
@@ -115,6 +117,7 @@ inline bool is_tc_precision(int p) { return p == FIO_PTF32 || p == FIO_PBF16 || 
 int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>& mdims, cudaStream_t s);
 size_t fx_scratch_bytes(fio_op op, int b, size_t elem);
 bool fx_takes(const fio::Stage& st, bool adj, bool wide, int b);
+int fft_build(fio_op op, cudaStream_t s);  // the DFT's twiddle table (fio_fft.cu)
 bool fx_all_wide(fio_op op);  // every stage of the operator has an FP64 digit copy
 bool fx_launch(const fio::Stage& st, bool adj, bool wide, const void* x, long long xrs, long long xcs, void* y,
                long long yrs, long long ycs, int b, void* scratch, size_t scratch_bytes, int* timeout, cudaStream_t s);
