@@ -1109,6 +1109,13 @@ bool inplace_split<float2>(const Stage& st, bool adj, float2* W, float2* P, long
   return true;
 }
 
+// Rows of a block up to which an in-place stage is written straight into the work vector: a block is
+// then one row tile of every stage kernel, whose CTA (or warp) has read all of the block's entries of
+// its right-hand sides before it writes any, and no other block reads them.  (Before, every HIF level
+// computed into scratch and copied back: 9 more launches of 2.5 us each in the 27 of the direct solve
+// at N = 1024.)
+constexpr int kDirectRows = kTileRows;
+
 // one INPLACE stage on the row-major work vector W (scratch S has the same shape; P, when not
 // null, is free scratch of pcap rows for the split variant)
 template <typename V>
@@ -1119,10 +1126,19 @@ void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, cudaStream_t s,
     mark(s);
     return;
   }
-  launch_stage<V>(st, adj, W, b, 1, S, b, 1, b, s);
-  const long long nidx = (long long)st.nblk * st.R;
-  const long long tot = nidx * b;
-  k_scatter_back<V><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(st.out, nidx, S, W, b);
+  // the fixed-point kernel reads W in a launch of its own (the gather), so it may write W
+  const int var = st.var[type_index<V>()][adj ? 1 : 0][rhs_bucket(b)];
+  if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, W, b, 1, W, b, 1, b, s, var == kFxVariant)) {
+    mark(s);
+    return;
+  }
+  const bool direct = std::max(st.maxcols[0], st.maxcols[1]) <= kDirectRows;
+  launch_stage<V>(st, adj, W, b, 1, direct ? W : S, b, 1, b, s);
+  if (!direct) {
+    const long long nidx = (long long)st.nblk * st.R;
+    const long long tot = nidx * b;
+    k_scatter_back<V><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(st.out, nidx, S, W, b);
+  }
   mark(s);
 }
 
@@ -1359,8 +1375,10 @@ extern "C" int fio_launch_count(fio_op op, int which, int b, int* launches) {
   if (!op || !launches || which < 0 || which > 3) return FIO_EINVAL;
   int bfl = 0, gl = 0;
   for (int k = 0; k < op->n_bf; ++k) bfl += op->st[k].nblk ? 1 : 0;
-  for (int k = op->n_bf; k < op->n_bf + op->n_hif; ++k) gl += op->st[k].nblk ? 4 : 0;
-  for (int k = op->n_bf + op->n_hif; k < (int)op->st.size(); ++k) gl += op->st[k].nblk ? 2 : 0;
+  // an in-place stage is one launch per direction, and a copy-back (or reduction) for large blocks
+  auto inplace = [&](int k) { return std::max(op->st[k].maxcols[0], op->st[k].maxcols[1]) <= kDirectRows ? 1 : 2; };
+  for (int k = op->n_bf; k < op->n_bf + op->n_hif; ++k) gl += op->st[k].nblk ? 2 * inplace(k) : 0;
+  for (int k = op->n_bf + op->n_hif; k < (int)op->st.size(); ++k) gl += op->st[k].nblk ? inplace(k) : 0;
   switch (which) {
     case 0:
     case 1: *launches = b ? bfl : 0; break;
