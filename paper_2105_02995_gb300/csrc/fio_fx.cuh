@@ -251,31 +251,42 @@ struct Acc96 {
   long long hi;
   uint32_t lo;
 };
-// v 2^s, rounded to nearest
+// v 2^s, rounded to nearest, in 32-bit integer steps (the FP64 pipe's two lanes a clock would take
+// four times as long for the conversion of a tile as its sums take to form)
 __device__ __forceinline__ double to_double(Acc96 v, int s) {
-  unsigned long long h = (unsigned long long)v.hi;
-  uint32_t l = v.lo;
-  const bool neg = v.hi < 0;
-  if (neg) {
-    l = 0u - l;
-    h = ~h + (l == 0u ? 1ull : 0ull);
+  uint32_t w2 = (uint32_t)((unsigned long long)v.hi >> 32), w1 = (uint32_t)v.hi, w0 = v.lo;
+  const uint32_t sg = (uint32_t)((int)w2 >> 31);
+  // magnitude: negated where the sign is set
+  asm("{\n\txor.b32 %0, %0, %3;\n\txor.b32 %1, %1, %3;\n\txor.b32 %2, %2, %3;\n\t"
+      "sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;\n\t}"
+      : "+r"(w0), "+r"(w1), "+r"(w2)
+      : "r"(sg));
+  int e = s + 95;  // exponent of w2's first bit
+  if (w2 == 0) {
+    w2 = w1;
+    w1 = w0;
+    w0 = 0;
+    e -= 32;
   }
-  int e = s + 32;  // exponent of h's last bit
-  if (h == 0) {
-    if (l == 0) return 0.0;
-    h = l;
-    l = 0;
-    e = s;
+  if (w2 == 0) {
+    w2 = w1;
+    w1 = 0;
+    e -= 32;
   }
-  const int lz = __clzll((long long)h);
-  if (lz) h = (h << lz) | (((unsigned long long)l << 32) >> (64 - lz));
-  e += 63 - lz;  // exponent of the leading bit
-  // 53 bits, to nearest (the carry of a mantissa of ones goes into the exponent)
-  const unsigned long long m = (h >> 11) + ((h >> 10) & 1ull);
-  const int be = e + 1023;
-  if (be < 1 || be > 2045) return neg ? -ldexp((double)m, e - 52) : ldexp((double)m, e - 52);
-  const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + m;
-  return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+  const int lz = __clz((int)w2);
+  const uint32_t h = __funnelshift_l(w1, w2, lz), l = __funnelshift_l(w0, w1, lz);
+  e -= lz;
+  // 53 of the 64 bits, to nearest (a carry out of a mantissa of ones goes into the exponent)
+  uint32_t mh = h >> 11, ml = __funnelshift_r(l, h, 11);
+  const uint32_t up = (l >> 10) & 1u;
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(ml), "+r"(mh) : "r"(up));
+  const int be = e + 1022;  // the leading bit adds the last 1
+  if (h == 0) return 0.0;
+  if (be < 0 || be > 2044) {
+    const double m = ldexp((double)(((unsigned long long)mh << 32) | ml), e - 52);
+    return sg ? -m : m;
+  }
+  return __hiloint2double((int)((mh + ((uint32_t)be << 20)) | (sg & 0x80000000u)), (int)ml);
 }
 // the upper 41 bits and the lower 23 converted apart: at most 2^-24 off before the last rounding
 // (the 64-bit conversion instruction is many times slower)
