@@ -493,6 +493,15 @@ template <> struct ChunkK<double2> { static constexpr int v = 16; };
 template <> struct ChunkK<float2> { static constexpr int v = 32; };
 template <> struct ChunkK<dfc> { static constexpr int v = 16; };
 
+// Stage launches whose CTAs are light enough to be started early (pdl_launch): complex multiply-adds
+// of a CTA's tile.  A 64 x 58 tile of 8 right-hand sides (30,000) gains 2.3 us a launch, one of
+// 64 x 228 x 32 (467,000) loses 15.
+constexpr long long kLightMacs = 110000;
+template <bool ADJ, typename V>
+bool light(const StageArgs<V>& a, int rows, int rhs) {
+  return (long long)rows * (ADJ ? a.R : a.C) * std::min(rhs, a.b) <= kLightMacs * a.ksplit;
+}
+
 template <typename V, bool ADJ, int TX, int TB, int TR>
 void launch_mm(StageArgs<V> a, cudaStream_t s) {
   constexpr int RT = (256 / TX) * TR, BT = TX * TB;
@@ -502,7 +511,7 @@ void launch_mm(StageArgs<V> a, cudaStream_t s) {
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + BT - 1) / BT));
-  k_stage_mm<V, ADJ, TX, TB, TR, ChunkK<V>::v><<<grid, 256, 0, s>>>(a);
+  pdl_launch(light<ADJ>(a, RT, BT), k_stage_mm<V, ADJ, TX, TB, TR, ChunkK<V>::v>, grid, 256, 0, s, a);
 }
 
 // Dynamic shared memory above 48 KB is opted into per kernel and per device: remember, per (device,
@@ -539,7 +548,7 @@ void launch_pipe(StageArgs<V> a, cudaStream_t s) {
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + S::BT - 1) / S::BT));
-  k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK><<<grid, 256, S::SMEM, s>>>(a);
+  pdl_launch(light<ADJ>(a, S::RT, S::BT), k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK>, grid, 256, S::SMEM, s, a);
 }
 // the same tiles with three real products per complex product (FP64 and double-float only)
 template <typename V, bool ADJ, int TX, int TB, int TR>
@@ -554,7 +563,7 @@ bool launch_pipe3(StageArgs<V> a, cudaStream_t s) {
     const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
     if (ncta == 0) return true;
     dim3 grid((unsigned)ncta, (unsigned)((a.b + S::BT - 1) / S::BT));
-    k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK, true><<<grid, 256, smem, s>>>(a);
+    pdl_launch(light<ADJ>(a, S::RT, S::BT), k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK, true>, grid, 256, smem, s, a);
     return true;
   } else {
     return false;
@@ -578,7 +587,7 @@ bool launch_vt(StageArgs<float2> a, cudaStream_t s) {
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return true;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + S::BT - 1) / S::BT), (unsigned)a.ksplit);
-  k_stage_mm_vt<ADJ, TX, TB, TR, NT, CK, MINB><<<grid, NT, S::SMEM, s>>>(a);
+  pdl_launch(light<ADJ>(a, S::RT, S::BT), k_stage_mm_vt<ADJ, TX, TB, TR, NT, CK, MINB>, grid, NT, S::SMEM, s, a);
   return true;
 }
 template <typename V, bool ADJ, int TX, int TB, int TR, int NT, int CK = 32,
@@ -605,7 +614,7 @@ bool launch_small(const StageArgs<V>& a, cudaStream_t s) {
     if (!smem_opt_in((const void*)k_stage_small<V, ADJ>, smem)) return false;
     if (a.nblk == 0) return true;
     dim3 grid((unsigned)((a.nblk + kSmallWarps - 1) / kSmallWarps), (unsigned)((a.b + 31) / 32));
-    k_stage_small<V, ADJ><<<grid, 32 * kSmallWarps, smem, s>>>(a);
+    pdl_launch(true, k_stage_small<V, ADJ>, grid, 32 * kSmallWarps, smem, s, a);
     return true;
   } else {
     return false;
@@ -632,7 +641,7 @@ bool launch_vec_b(StageArgs<V> a, cudaStream_t s) {
   a.ntiles = (nrows + kTileRows - 1) / kTileRows;
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return true;
-  k_stage_vec<V, ADJ, B><<<(unsigned)ncta, 256, (size_t)need, s>>>(a);
+  pdl_launch(light<ADJ>(a, kTileRows, B), k_stage_vec<V, ADJ, B>, (unsigned)ncta, 256, (size_t)need, s, a);
   return true;
 }
 template <typename V, bool ADJ>
@@ -770,7 +779,7 @@ void launch_tc_dir(const TcArgs& a, int ncta, cudaStream_t s) {
   const int need = tc_smem_bytes(MODE, a.nmax, a.ncmax);
   smem_opt_in((const void*)k_stage_tc<ADJ, MODE>, need);
   dim3 grid((unsigned)ncta, (unsigned)((a.b + kTcMaxRhs - 1) / kTcMaxRhs));
-  k_stage_tc<ADJ, MODE><<<grid, 128, need, s>>>(a);
+  pdl_launch((long long)kTcRows * a.ncmax * a.b <= kLightMacs, k_stage_tc<ADJ, MODE>, grid, 128, need, s, a);
 }
 
 // the ring variant with S stages; false when its shared memory does not fit
@@ -780,7 +789,7 @@ bool launch_tc_ring(const TcArgs& a, int ncta, cudaStream_t s) {
   if (need > 227 * 1024) return false;
   if (!smem_opt_in((const void*)k_stage_tc_ring<ADJ, MODE, S>, need)) return false;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + kTcMaxRhs - 1) / kTcMaxRhs));
-  k_stage_tc_ring<ADJ, MODE, S><<<grid, 192, need, s>>>(a);
+  pdl_launch(false, k_stage_tc_ring<ADJ, MODE, S>, grid, 192, need, s, a);
   return true;
 }
 
@@ -879,7 +888,7 @@ bool launch_tma(const Stage& st, bool adj, const float2* x, long long xrs, long 
 #define FIO_TMA_CASE(MODE, ADJ)                                                                   \
   case 2 * MODE + ADJ:                                                                            \
     if (!smem_opt_in((const void*)k_stage_tma<ADJ, MODE>, need)) return false;                   \
-    k_stage_tma<ADJ, MODE><<<grid, tma::kThreads, need, s>>>(a, map);                             \
+    pdl_launch(false, k_stage_tma<ADJ, MODE>, grid, tma::kThreads, need, s, a, map);                             \
     return true;
     FIO_TMA_CASE(kTcTF32, 0)
     FIO_TMA_CASE(kTcTF32, 1)
@@ -1081,7 +1090,7 @@ bool inplace_split_fp32(const Stage& st, bool adj, float2* W, float2* P, long lo
   const bool ok = adj ? launch_vt<true, 8, 4, 8, 128, 16>(a, s) : launch_vt<false, 8, 4, 8, 128, 16>(a, s);
   if (!ok) return false;
   const long long tot = prow * b;
-  k_partial_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(P, a.ksplit, prow, b, st.out, W);
+  pdl_launch(true, k_partial_reduce, (unsigned)((tot + 255) / 256), 256, 0, s, P, a.ksplit, prow, b, st.out, W);
   return true;
 }
 
@@ -1105,7 +1114,7 @@ bool inplace_split<float2>(const Stage& st, bool adj, float2* W, float2* P, long
   ks = std::max(1, std::min(ks, 64));
   if (!launch_tma(st, adj, W, b, 1, nullptr, 0, 0, b, s, kTmaVariant, ks, P, 0)) return false;
   const long long tot = prow * b;
-  k_partial_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(P, ks, prow, b, st.out, W);
+  pdl_launch(true, k_partial_reduce, (unsigned)((tot + 255) / 256), 256, 0, s, P, ks, prow, b, st.out, W);
   return true;
 }
 
@@ -1137,7 +1146,7 @@ void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, cudaStream_t s,
   if (!direct) {
     const long long nidx = (long long)st.nblk * st.R;
     const long long tot = nidx * b;
-    k_scatter_back<V><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(st.out, nidx, S, W, b);
+    pdl_launch(true, k_scatter_back<V>, (unsigned)((tot + 255) / 256), 256, 0, s, st.out, nidx, S, W, b);
   }
   mark(s);
 }
@@ -1145,13 +1154,13 @@ void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, cudaStream_t s,
 template <typename V>
 void to_row(const V* X, long long ld, V* W, long long N, int b, cudaStream_t s) {
   dim3 grid((unsigned)((N + 31) / 32), (unsigned)((b + 31) / 32));
-  k_col_to_row<V><<<grid, dim3(32, 8), 0, s>>>(X, ld, W, N, b);
+  pdl_launch(true, k_col_to_row<V>, grid, dim3(32, 8), 0, s, X, ld, W, N, b);
   mark(s);
 }
 template <typename V>
 void to_col(const V* W, V* Y, long long ld, long long N, int b, cudaStream_t s) {
   dim3 grid((unsigned)((N + 31) / 32), (unsigned)((b + 31) / 32));
-  k_row_to_col<V><<<grid, dim3(32, 8), 0, s>>>(W, Y, ld, N, b);
+  pdl_launch(true, k_row_to_col<V>, grid, dim3(32, 8), 0, s, W, Y, ld, N, b);
   mark(s);
 }
 
@@ -1258,9 +1267,9 @@ int apply_df(fio_op op, Which w, const void* xv, void* yv, int64_t ld, int b, cu
   dfc *X = (dfc*)bufs[3], *Y = (dfc*)bufs[4];
   const long long n = op->N * (long long)b;
   const unsigned g = (unsigned)((n + 255) / 256);
-  k_c128_to_df<<<g, 256, 0, s>>>((const double2*)xv, ld, X, op->N, b);
+  pdl_launch(true, k_c128_to_df, g, 256, 0, s, (const double2*)xv, ld, X, op->N, b);
   apply_core<dfc>(op, w, X, Y, op->N, b, (dfc*)bufs[0], (dfc*)bufs[1], (dfc*)bufs[2], s);
-  k_df_to_c128<<<g, 256, 0, s>>>(Y, op->N, (double2*)yv, ld, b);
+  pdl_launch(true, k_df_to_c128, g, 256, 0, s, Y, op->N, (double2*)yv, ld, b);
   return finish(s);
 }
 

@@ -210,6 +210,8 @@ template <typename R, int SIGN>
 __global__ void __launch_bounds__(kFftThreads) k_fft_pass(FftPass p) {
   using V = typename Cplx<R>::T;
   __shared__ V s[kFftShared];
+  fio::pdl_go();
+  fio::pdl_wait();
   const int t0 = blockIdx.x * (kFftElems / p.L);
   const V* x = reinterpret_cast<const V*>(p.x) + (long long)blockIdx.y * p.ldx;
   V* y = reinterpret_cast<V*>(p.y) + (long long)blockIdx.y * p.ldy;
@@ -246,8 +248,8 @@ template <typename R>
 int run_pass(const FftPass& p, bool inverse, int b, cudaStream_t s) {
   const int TT = kFftElems / p.L;
   dim3 grid((unsigned)((p.T + TT - 1) / TT), (unsigned)b);
-  if (inverse) k_fft_pass<R, 1><<<grid, kFftThreads, 0, s>>>(p);
-  else k_fft_pass<R, -1><<<grid, kFftThreads, 0, s>>>(p);
+  if (inverse) pdl_launch(true, k_fft_pass<R, 1>, grid, kFftThreads, 0, s, p);
+  else pdl_launch(true, k_fft_pass<R, -1>, grid, kFftThreads, 0, s, p);
   return FIO_OK;
 }
 

@@ -92,6 +92,7 @@ struct FxArgs {
   long long yrs, ycs;
   int b;
   int nraw;           // raw ring slots (2 .. kMaxRaw)
+  long long steps;    // K steps of all units (host side)
   int* timeout;       // set when a bounded wait gave up
 };
 
@@ -317,8 +318,10 @@ __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, i
   const int* cidx = a.colidx + (size_t)blk * a.lcol;
   const V* x = (const V*)a.x;
   const int tid = threadIdx.x;
+  pdl_go();
   if (tid < BT) s_mag[tid] = s_low[tid] = 0u;
   __syncthreads();
+  pdl_wait();
   // lanes along the right-hand sides (BT a power of two; those beyond wt idle)
   const int j = tid % BT, c0 = tid / BT;
   constexpr int CS = 256 / BT;
@@ -425,6 +428,7 @@ __global__ void __launch_bounds__(fx::kThreads, 1) k_stage_fx(const FxArgs a) {
   __syncthreads();
   fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+  pdl_go();  // only now: a kernel started behind this one may hold tensor memory while it waits for it
   bool ok = true;
 
   if (warp < kDrainWarps) {
@@ -441,6 +445,7 @@ __global__ void __launch_bounds__(fx::kThreads, 1) k_stage_fx(const FxArgs a) {
       ejl = lane < BT / 2 && jl < a.b ? a.ej[(size_t)e.blk * a.b + jl] : 0;
     };
     FxUnit nx = unit(blockIdx.x);
+    pdl_wait();
     row_of(nx, blockIdx.x);
     for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
       const FxUnit e = nx;
@@ -622,6 +627,7 @@ __global__ void __launch_bounds__(fx::kThreads, 1) k_stage_fx(const FxArgs a) {
           expect(full, abytes + xbytes);
           if (a.nrt == 1) bulk(dst, A, abytes, full, pol);
           else bulk(dst, A, abytes, full);
+          if (ic == 0) pdl_wait();  // the factor's first chunk does not wait for the vector
           bulk(dst + 16384, X, xbytes, full);
           A += abytes;
           X += xbytes;

@@ -26,6 +26,8 @@
 
 #include <type_traits>
 
+#include "fio_internal.h"
+
 namespace fio {
 
 __device__ __forceinline__ double2 cmac(double2 acc, double2 a, double2 b) {
@@ -220,6 +222,8 @@ __global__ void __launch_bounds__(256) k_stage_mm(StageArgs<V> a) {
   const int tx = tid % TX;
   const int ty = tid / TX;
 
+  pdl_go();
+  pdl_wait();
   V acc[TR][TB];
 #pragma unroll
   for (int i = 0; i < TR; ++i)
@@ -392,7 +396,8 @@ __global__ void __launch_bounds__(256) k_stage_mm_pipe(StageArgs<V> a) {
   const int tx = tid % TX;
   const int ty = tid / TX;
 
-  auto load = [&](int buf, int c0) {
+  pdl_go();
+  auto load = [&](int buf, int c0, bool first = false) {
     V* dM = sM + buf * MROWS * MLD;
     constexpr int CPR = MCOLS / VPC;
     for (int e = tid; e < MROWS * CPR; e += 256) {
@@ -405,6 +410,7 @@ __global__ void __launch_bounds__(256) k_stage_mm_pipe(StageArgs<V> a) {
       cp_async16(dM + mr * MLD + mc, ok ? (const void*)(M + (size_t)grow * a.C + gcol) : (const void*)M,
                  ok ? 16 : 0);
     }
+    if (first) pdl_wait();  // the factor's first chunk does not wait for the vector
     V* dX = sX + buf * CK * BT;
     constexpr int CPX = BT / VPC;
     for (int e = tid; e < CK * CPX; e += 256) {
@@ -440,7 +446,7 @@ __global__ void __launch_bounds__(256) k_stage_mm_pipe(StageArgs<V> a) {
   }
 
   const int nchunks = (ncols + CK - 1) / CK;
-  load(0, 0);
+  load(0, 0, true);
   for (int k = 0; k < nchunks; ++k) {
     if (k + 1 < nchunks) {
       load((k + 1) & 1, (k + 1) * CK);
@@ -596,7 +602,8 @@ __global__ void __launch_bounds__(NT, MINB) k_stage_mm_vt(StageArgs<float2> a) {
       nidx[u] = (e < CK * CPX && c < ncols) ? colidx[c] : -1;
     }
   };
-  auto load = [&](int buf, int c0) {
+  pdl_go();
+  auto load = [&](int buf, int c0, bool first = false) {
     float2* dM = sM + buf * MTILE;
     constexpr int CPR = MCOLS / 2;
     for (int e = tid; e < MROWS * CPR; e += NT) {
@@ -608,6 +615,7 @@ __global__ void __launch_bounds__(NT, MINB) k_stage_mm_vt(StageArgs<float2> a) {
       cp_async16(dM + S::mofs(mr, mc), ok ? (const void*)(M + (size_t)grow * a.C + gcol) : (const void*)M,
                  ok ? 16 : 0);
     }
+    if (first) pdl_wait();  // the factor's first chunk does not wait for the vector
     float2* dX = sX + buf * XTILE;
 #pragma unroll
     for (int u = 0; u < NXP; ++u) {
@@ -639,7 +647,9 @@ __global__ void __launch_bounds__(NT, MINB) k_stage_mm_vt(StageArgs<float2> a) {
   const int nchunks = min(nch, kb + cps) - kb;
   if (nchunks > 0) {
     fetch_idx(kb * CK);
-    load(0, kb * CK);
+    load(0, kb * CK, true);
+  } else {
+    pdl_wait();
   }
   for (int k = 0; k < nchunks; ++k) {
     if (k + 1 < nchunks) {
@@ -712,6 +722,7 @@ __global__ void __launch_bounds__(32 * kSmallWarps) k_stage_small(StageArgs<V> a
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int blk = blockIdx.x * kSmallWarps + w;
+  pdl_go();
   if (blk >= a.nblk) return;  // warp-uniform; the kernel has no CTA-wide barrier
   const int RC = a.R * a.C, cmax = ADJ ? a.R : a.C;
   V* sm = reinterpret_cast<V*>(smem_raw) + (size_t)w * (RC + 32 * cmax);
@@ -728,6 +739,7 @@ __global__ void __launch_bounds__(32 * kSmallWarps) k_stage_small(StageArgs<V> a
   const int* rowidx = ADJ ? a.in + (size_t)blk * a.C : a.out + (size_t)blk * a.R;
   const int* colidx = ADJ ? a.out + (size_t)blk * a.R : a.in + (size_t)blk * a.C;
   for (int e = lane; e < RC; e += 32) sm[e] = M[e];
+  pdl_wait();
   const int j = blockIdx.y * 32 + lane;
   const bool on = j < a.b;
 #pragma unroll 4
@@ -814,9 +826,12 @@ __global__ void __launch_bounds__(256) k_stage_vec(StageArgs<V> a) {
   const int* colidx = ADJ ? a.out + (size_t)blk * a.R : a.in + (size_t)blk * a.C;
   const int r0 = tile * 64;
   const int tid = threadIdx.x;
+  pdl_go();
+  int idx = tid < ncols * B ? colidx[tid % ncols] : -1;
+  pdl_wait();
   for (int e = tid; e < ncols * B; e += 256) {
     const int j = e / ncols, c = e - j * ncols;
-    const int idx = colidx[c];
+    if (e != tid) idx = colidx[c];
     sX[e] = idx >= 0 ? a.x[(long long)idx * a.xrs + (long long)j * a.xcs] : czero<V>();
   }
   __syncthreads();
@@ -875,6 +890,8 @@ __global__ void __launch_bounds__(256) k_stage_vec(StageArgs<V> a) {
 // block has already overwritten.
 template <typename V>
 __global__ void k_scatter_back(const int* idx, long long nidx, const V* S, V* W, int b) {
+  pdl_go();
+  pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nidx * b) return;
   const long long k = t / b;
@@ -887,6 +904,8 @@ __global__ void k_scatter_back(const int* idx, long long nidx, const V* S, V* W,
 // column-major (ld) <-> row-major (b) layout changes of an N x b array, 32 x 32 smem tiles
 template <typename V>
 __global__ void k_col_to_row(const V* X, long long ld, V* W, long long N, int b) {
+  pdl_go();
+  pdl_wait();
   __shared__ V t[32][33];
   const long long i0 = (long long)blockIdx.x * 32;
   const int j0 = blockIdx.y * 32;
@@ -905,6 +924,8 @@ __global__ void k_col_to_row(const V* X, long long ld, V* W, long long N, int b)
 
 template <typename V>
 __global__ void k_row_to_col(const V* W, V* Y, long long ld, long long N, int b) {
+  pdl_go();
+  pdl_wait();
   __shared__ V t[32][33];
   const long long i0 = (long long)blockIdx.x * 32;
   const int j0 = blockIdx.y * 32;
@@ -937,12 +958,16 @@ static __global__ void k_split_df(const double2* a, dfc* b, size_t n) {
 }
 // N x b column-major complex128 (leading dimension ld) -> double-float (leading dimension N), and back
 static __global__ void k_c128_to_df(const double2* x, long long ld, dfc* y, long long N, int b) {
+  pdl_go();
+  pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const long long j = t / N, i = t - j * N;
   y[t] = split_df(x[j * ld + i]);
 }
 static __global__ void k_df_to_c128(const dfc* y, long long N, double2* x, long long ld, int b) {
+  pdl_go();
+  pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const long long j = t / N, i = t - j * N;

@@ -30,6 +30,8 @@ constexpr int kRedThreads = 512;
 // out[j] = sum_i conj(a[i, j]) b[i, j]   (one CTA per column j, fixed reduction tree)
 __global__ void k_coldot(const double2* a, const double2* b, long long N, long long lda,
                          long long ldb, double2* out) {
+  fio::pdl_go();
+  fio::pdl_wait();
   __shared__ double sr[kRedThreads], si[kRedThreads];
   const int j = blockIdx.x;
   const double2* x = a + (long long)j * lda;
@@ -56,6 +58,8 @@ __global__ void k_coldot(const double2* a, const double2* b, long long N, long l
 // H[i + (k+1) j] = <V_i[:, j], w[:, j]> for i <= k   (grid (k+1, b))
 __global__ void k_basisdot(const double2* V, long long vstride, const double2* w, long long N,
                            int b, int kp1, double2* H) {
+  fio::pdl_go();
+  fio::pdl_wait();
   __shared__ double sr[kRedThreads], si[kRedThreads];
   const int i = blockIdx.x, j = blockIdx.y;
   const double2* x = V + (long long)i * vstride + (long long)j * N;
@@ -82,6 +86,8 @@ __global__ void k_basisdot(const double2* V, long long vstride, const double2* w
 // w[:, j] -= sum_{i<=k} H[i + kp1 j] V_i[:, j]
 __global__ void k_basis_sub(const double2* V, long long vstride, double2* w, long long N, int b,
                             int kp1, const double2* H) {
+  fio::pdl_go();
+  fio::pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const int j = (int)(t / N);
@@ -99,6 +105,8 @@ __global__ void k_basis_sub(const double2* V, long long vstride, double2* w, lon
 // y[:, j] = alpha[j] x[:, j] + beta[j] y[:, j]   (x, y with leading dimensions)
 __global__ void k_axpby(const double2* alpha, const double2* x, long long ldx, const double2* beta,
                         double2* y, long long ldy, long long N, int b) {
+  fio::pdl_go();
+  fio::pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const int j = (int)(t / N);
@@ -112,10 +120,14 @@ __global__ void k_axpby(const double2* alpha, const double2* x, long long ldx, c
 }
 
 __global__ void k_to32(const double2* x, float2* y, long long n) {
+  fio::pdl_go();
+  fio::pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < n) y[t] = make_float2((float)x[t].x, (float)x[t].y);
 }
 __global__ void k_add32(const float2* d, double2* f, long long ldf, long long N, int b) {
+  fio::pdl_go();
+  fio::pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const int j = (int)(t / N);
@@ -180,7 +192,7 @@ struct Ctx {
 
 int dots(Ctx& c, const double2* a, long long lda, const double2* bb, long long ldb, double2* out_dev,
          std::vector<double2>* host) {
-  k_coldot<<<c.b, kRedThreads, 0, c.s>>>(a, bb, c.N, lda, ldb, out_dev);
+  pdl_launch(true, k_coldot, c.b, kRedThreads, 0, c.s, a, bb, c.N, lda, ldb, out_dev);
   if (host) {
     host->resize(c.b);
     if (cudaMemcpyAsync(host->data(), out_dev, c.b * sizeof(double2), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
@@ -195,7 +207,7 @@ int axpby(Ctx& c, const std::vector<double2>& al, const double2* x, long long ld
   double2* d = c.dsc;
   cudaMemcpyAsync(d, al.data(), c.b * sizeof(double2), cudaMemcpyHostToDevice, c.s);
   cudaMemcpyAsync(d + c.b, be.data(), c.b * sizeof(double2), cudaMemcpyHostToDevice, c.s);
-  k_axpby<<<nblocks(c.N * c.b), 256, 0, c.s>>>(d, x, ldx, d + c.b, y, ldy, c.N, c.b);
+  pdl_launch(true, k_axpby, nblocks(c.N * c.b), 256, 0, c.s, d, x, ldx, d + c.b, y, ldy, c.N, c.b);
   // the host vectors may change right after: make the copies complete first
   return cudaStreamSynchronize(c.s) == cudaSuccess ? FIO_OK : FIO_ECUDA;
 }
@@ -212,11 +224,11 @@ inline double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 int precond(Ctx& c, Work& w, int which, const double2* x, double2* y, int prec) {
   if (prec == FIO_P64) return fio_apply_internal(c.op, which, x, y, c.N, c.b, FIO_P64, c.s);
   const long long n = c.N * c.b;
-  k_to32<<<nblocks(n), 256, 0, c.s>>>(x, w.v32[0], n);
+  pdl_launch(true, k_to32, nblocks(n), 256, 0, c.s, x, w.v32[0], n);
   int rc = fio_apply_internal(c.op, which, w.v32[0], w.v32[1], c.N, c.b, prec, c.s);
   if (rc) return rc;
   cudaMemsetAsync(y, 0, n * sizeof(double2), c.s);
-  k_add32<<<nblocks(n), 256, 0, c.s>>>(w.v32[1], y, c.N, c.N, c.b);
+  pdl_launch(true, k_add32, nblocks(n), 256, 0, c.s, w.v32[1], y, c.N, c.N, c.b);
   return cudaGetLastError() == cudaSuccess ? FIO_OK : FIO_ECUDA;
 }
 
@@ -422,8 +434,8 @@ extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b,
         std::vector<double2> h1((size_t)(k + 1) * b), h2((size_t)(k + 1) * b);
         for (int pass = 0; pass < 2; ++pass) {
           dim3 grid(k + 1, b);
-          k_basisdot<<<grid, kRedThreads, 0, s>>>(V, vs, Wv, N, b, k + 1, w.Hd);
-          k_basis_sub<<<nblocks(N * b), 256, 0, s>>>(V, vs, Wv, N, b, k + 1, w.Hd);
+          pdl_launch(true, k_basisdot, grid, kRedThreads, 0, s, V, vs, Wv, N, b, k + 1, w.Hd);
+          pdl_launch(true, k_basis_sub, nblocks(N * b), 256, 0, s, V, vs, Wv, N, b, k + 1, w.Hd);
           auto& dst = pass ? h2 : h1;
           if (cudaMemcpyAsync(dst.data(), w.Hd, (size_t)(k + 1) * b * sizeof(double2), cudaMemcpyDeviceToHost, s) != cudaSuccess)
             return FIO_ECUDA;
@@ -502,7 +514,7 @@ extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b,
       for (auto& v : coef) v = make_double2(-v.x, -v.y);
       cudaMemsetAsync(Zt, 0, (size_t)N * b * sizeof(double2), s);
       cudaMemcpyAsync(w.Hd, coef.data(), coef.size() * sizeof(double2), cudaMemcpyHostToDevice, s);
-      if (k > 0) k_basis_sub<<<nblocks(N * b), 256, 0, s>>>(V, vs, Zt, N, b, k, w.Hd);
+      if (k > 0) pdl_launch(true, k_basis_sub, nblocks(N * b), 256, 0, s, V, vs, Zt, N, b, k, w.Hd);
       rc = precond(c, w, 3, Zt, Wv, opts->inner);
       if (rc) return rc;
       std::vector<double2> one(b, make_double2(1, 0));

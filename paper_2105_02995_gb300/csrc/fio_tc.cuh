@@ -34,6 +34,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fio_internal.h"
+
 namespace fio {
 
 __device__ int g_tc_timeout;  // set when a bounded wait in k_stage_tc gave up
@@ -235,6 +237,8 @@ __global__ void __launch_bounds__(128) k_stage_tc(TcArgs a) {
   __syncthreads();
   fence_after();
   const uint32_t tmem = s_tmem;
+  pdl_go();  // only now: a kernel started behind this one may hold tensor memory while it waits for it
+  pdl_wait();
 
   bool ok = true;
   for (int k = 0; k < nchunks && ok; ++k) {
@@ -459,6 +463,8 @@ __global__ void __launch_bounds__(192) k_stage_tc_ring(TcArgs a) {
   __syncthreads();
   fence_after();
   const uint32_t tmem = s_tmem;
+  pdl_go();  // only now: a kernel started behind this one may hold tensor memory while it waits for it
+  pdl_wait();
 
   bool ok = true;
   if (warp == 4) {

@@ -207,6 +207,8 @@ __global__ void __launch_bounds__(tma::kThreads, 1) k_stage_tma(const TmaArgs a,
   __syncthreads();
   fence_after();
   const uint32_t tmem = s_tmem;
+  pdl_go();  // only now: a kernel started behind this one may hold tensor memory while it waits for it
+  pdl_wait();
   bool ok = true;
 
   if (warp == 0) {
@@ -516,6 +518,8 @@ __global__ void __launch_bounds__(tma::kThreads, 1) k_stage_tma(const TmaArgs a,
 // the block rows' own indices (the in-place stage's copy-back): W[idx[r]][j] = sum_ks part[ks][r][j]
 // for every packed row r of the stage with idx[r] >= 0 (the blocks' index sets are disjoint).
 __global__ void k_partial_reduce(const float2* part, int ksplit, long long prow, int b, const int* idx, float2* W) {
+  pdl_go();
+  pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= prow * b) return;
   const long long r = t / b;
