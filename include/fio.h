@@ -179,6 +179,7 @@ int fio_apply_inv_host(fio_op op, const void* u_host, void* f_host, int64_t ld, 
  *   FIO_IR      iterative refinement: residual r = u - K-dot f on complex128 vectors in
  *               opts->outer precision (FP64 or double-float), correction G-dot K-dot* r in
  *               opts->inner precision, FP64 update f += d.
+ * (FIO_PTF32X3 as the inner precision runs as FIO_P32: closer to the factors' product, and faster.)
  * Every method computes its true residuals u - K-dot f in opts->outer precision (PCG and GMRES
  * run their Krylov products in FP64 whatever opts->outer is).  With opts->residual_op (FIO_IR,
  * FIO_DIRECT) those residuals, and hence tol and info->relres, refer to that operator's K-dot:

@@ -407,6 +407,7 @@ extern "C" int fio_release(fio_op op) {
   if (op->fft_tw) cudaFree(op->fft_tw);
   if (op->arena_tc) cudaFree(op->arena_tc);
   if (op->scratch) cudaFree(op->scratch);
+  if (op->flag_host) cudaFreeHost(op->flag_host);
   fio_solver_free(op);
   cudaGetLastError();
   delete op;
@@ -1319,6 +1320,20 @@ int fio_tc_timeout_reset() {
   return v;
 }
 
+int fio_sync_flag(fio_op op, cudaStream_t s) {
+  if (!op->flag_host) {
+    if (cudaMallocHost(&op->flag_host, sizeof(int)) != cudaSuccess) {
+      cudaGetLastError();
+      op->flag_host = nullptr;
+    }
+  }
+  if (!op->flag_host) return cudaStreamSynchronize(s) == cudaSuccess ? fio_tc_timeout_reset() : -1;
+  if (cudaMemcpyFromSymbolAsync(op->flag_host, g_tc_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return -1;
+  return *op->flag_host ? fio_tc_timeout_reset() : 0;
+}
+
 extern "C" int fio_apply_K(fio_op op, const void* x, void* y, int64_t ld, int b, int dtype,
                            int precision, void* stream) {
   return apply_any(op, W_K, x, y, ld, b, dtype, precision, stream);
@@ -1364,10 +1379,9 @@ extern "C" int fio_apply_inv_host(fio_op op, const void* u_host, void* f_host, i
       ? cudaMemcpyAsync(f_host, F, w * (size_t)b, cudaMemcpyDeviceToHost, s)
       : cudaMemcpy2DAsync(f_host, (size_t)ld * es, F, w, w, (size_t)b, cudaMemcpyDeviceToHost, s);
   if (e_out != cudaSuccess) return FIO_ECUDA;
-  if (cudaStreamSynchronize(s) != cudaSuccess) return FIO_ECUDA;
   // a tensor-core bounded wait that gave up left part of f unwritten: report it here, at the
   // call that produced the result, not at some later synchronising call
-  const int to = fio_tc_timeout_reset();
+  const int to = fio_sync_flag(op, s);
   return to < 0 ? FIO_ECUDA : (to > 0 ? FIO_ETIMEOUT : FIO_OK);
 }
 

@@ -107,6 +107,9 @@ struct fio_op_s {
   size_t fft_bytes = 0;
   void* solver = nullptr;         // solver work arrays (fio_solve.cu)
   size_t solver_bytes = 0;
+  int* flag_host = nullptr;       // pinned copy of the timeout flag (fio_sync_flag)
+  void* solver_host = nullptr;    // pinned scalars that the solver's kernels write and the host reads
+  size_t solver_host_bytes = 0;
 };
 
 // Kernels of an apply or a solve are launched with programmatic stream serialisation where `early`:
@@ -165,3 +168,5 @@ void fio_solver_free(fio_op op);
 // 1 when a tensor-core kernel's bounded wait gave up since the last call (and clear the flag),
 // 0 otherwise, -1 on a CUDA error
 int fio_tc_timeout_reset();
+// synchronise s with the flag read back in the same wait (a copy of its own takes 8 us); as above
+int fio_sync_flag(fio_op op, cudaStream_t s);

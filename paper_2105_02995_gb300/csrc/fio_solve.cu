@@ -18,6 +18,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "fio.h"
@@ -28,8 +29,9 @@ namespace {
 constexpr int kRedThreads = 512;
 
 // out[j] = sum_i conj(a[i, j]) b[i, j]   (one CTA per column j, fixed reduction tree)
+// (host: pinned memory that the host reads after a synchronise, or null)
 __global__ void k_coldot(const double2* a, const double2* b, long long N, long long lda,
-                         long long ldb, double2* out) {
+                         long long ldb, double2* out, double2* host) {
   fio::pdl_go();
   fio::pdl_wait();
   __shared__ double sr[kRedThreads], si[kRedThreads];
@@ -52,12 +54,15 @@ __global__ void k_coldot(const double2* a, const double2* b, long long N, long l
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[j] = make_double2(sr[0], si[0]);
+  if (threadIdx.x == 0) {
+    out[j] = make_double2(sr[0], si[0]);
+    if (host) host[j] = make_double2(sr[0], si[0]);
+  }
 }
 
 // H[i + (k+1) j] = <V_i[:, j], w[:, j]> for i <= k   (grid (k+1, b))
 __global__ void k_basisdot(const double2* V, long long vstride, const double2* w, long long N,
-                           int b, int kp1, double2* H) {
+                           int b, int kp1, double2* H, double2* host) {
   fio::pdl_go();
   fio::pdl_wait();
   __shared__ double sr[kRedThreads], si[kRedThreads];
@@ -80,7 +85,10 @@ __global__ void k_basisdot(const double2* V, long long vstride, const double2* w
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) H[i + (long long)kp1 * j] = make_double2(sr[0], si[0]);
+  if (threadIdx.x == 0) {
+    H[i + (long long)kp1 * j] = make_double2(sr[0], si[0]);
+    host[i + (long long)kp1 * j] = make_double2(sr[0], si[0]);
+  }
 }
 
 // w[:, j] -= sum_{i<=k} H[i + kp1 j] V_i[:, j]
@@ -102,16 +110,21 @@ __global__ void k_basis_sub(const double2* V, long long vstride, double2* w, lon
   w[t] = acc;
 }
 
-// y[:, j] = alpha[j] x[:, j] + beta[j] y[:, j]   (x, y with leading dimensions)
-__global__ void k_axpby(const double2* alpha, const double2* x, long long ldx, const double2* beta,
-                        double2* y, long long ldy, long long N, int b) {
+// y[:, j] = alpha[j] x[:, j] + beta[j] y[:, j]   (x, y with leading dimensions), the scalars of up to
+// kCoefs columns as launch parameters: no copy, and nothing for the host to wait for
+constexpr int kCoefs = 96;
+struct Coefs {
+  double2 a[kCoefs], b[kCoefs];
+};
+__global__ void k_axpby(const __grid_constant__ Coefs q, const double2* x, long long ldx, double2* y, long long ldy,
+                        long long N, int b) {
   fio::pdl_go();
   fio::pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= N * b) return;
   const int j = (int)(t / N);
   const long long i = t - (long long)j * N;
-  const double2 a = alpha[j], bb = beta[j];
+  const double2 a = q.a[j], bb = q.b[j];
   const double2 xv = x[i + j * ldx], yv = y[i + j * ldy];
   double2 r;
   r.x = a.x * xv.x - a.y * xv.y + bb.x * yv.x - bb.y * yv.y;
@@ -144,6 +157,7 @@ struct Work {
   double2* Hd;         // (restart + 1) x b scalars
   double2* sc;         // 4 x b scalars
   float2* v32[2];      // N x b
+  double2* host;       // pinned, 2 (restart + 1) x b scalars: what the kernels hand to the host
 };
 
 int get_work(fio_op op, int b, int restart, Work* w) {
@@ -161,6 +175,18 @@ int get_work(fio_op op, int b, int restart, Work* w) {
     }
     op->solver_bytes = need;
   }
+  const size_t hneed = (2 * (size_t)(restart + 1) * b + 2 * (size_t)b) * sizeof(double2);
+  if (hneed > op->solver_host_bytes) {
+    if (op->solver_host) cudaFreeHost(op->solver_host);
+    op->solver_host = nullptr;
+    op->solver_host_bytes = 0;
+    if (cudaMallocHost(&op->solver_host, hneed) != cudaSuccess) {
+      cudaGetLastError();
+      return FIO_ENOMEM;
+    }
+    op->solver_host_bytes = hneed;
+  }
+  w->host = (double2*)op->solver_host;
   uint8_t* p = (uint8_t*)op->solver;
   for (int k = 0; k < 6; ++k) {
     w->v[k] = (double2*)p;
@@ -185,31 +211,34 @@ struct Ctx {
   long long N;
   int b;
   cudaStream_t s;
-  double2* dsc;         // device scalar scratch (4 x b)
+  double2* host;        // pinned scalars (dots)
   int outer = FIO_P64;  // precision of the true residuals (FIO_P64 or FIO_PDF)
   bool f_zero = false;  // f is known to be zero (the next residual is u itself)
 };
 
 int dots(Ctx& c, const double2* a, long long lda, const double2* bb, long long ldb, double2* out_dev,
          std::vector<double2>* host) {
-  pdl_launch(true, k_coldot, c.b, kRedThreads, 0, c.s, a, bb, c.N, lda, ldb, out_dev);
+  pdl_launch(true, k_coldot, c.b, kRedThreads, 0, c.s, a, bb, c.N, lda, ldb, out_dev, c.host);
   if (host) {
-    host->resize(c.b);
-    if (cudaMemcpyAsync(host->data(), out_dev, c.b * sizeof(double2), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
-        cudaStreamSynchronize(c.s) != cudaSuccess)
-      return FIO_ECUDA;
+    if (cudaStreamSynchronize(c.s) != cudaSuccess) return FIO_ECUDA;
+    host->assign(c.host, c.host + c.b);
   }
   return cudaGetLastError() == cudaSuccess ? FIO_OK : FIO_ECUDA;
 }
 
 int axpby(Ctx& c, const std::vector<double2>& al, const double2* x, long long ldx,
           const std::vector<double2>& be, double2* y, long long ldy) {
-  double2* d = c.dsc;
-  cudaMemcpyAsync(d, al.data(), c.b * sizeof(double2), cudaMemcpyHostToDevice, c.s);
-  cudaMemcpyAsync(d + c.b, be.data(), c.b * sizeof(double2), cudaMemcpyHostToDevice, c.s);
-  pdl_launch(true, k_axpby, nblocks(c.N * c.b), 256, 0, c.s, d, x, ldx, d + c.b, y, ldy, c.N, c.b);
-  // the host vectors may change right after: make the copies complete first
-  return cudaStreamSynchronize(c.s) == cudaSuccess ? FIO_OK : FIO_ECUDA;
+  for (int j0 = 0; j0 < c.b; j0 += kCoefs) {
+    const int nb = std::min(kCoefs, c.b - j0);
+    Coefs q;
+    for (int j = 0; j < nb; ++j) {
+      q.a[j] = al[j0 + j];
+      q.b[j] = be[j0 + j];
+    }
+    pdl_launch(true, k_axpby, nblocks(c.N * nb), 256, 0, c.s, q, x + (long long)j0 * ldx, ldx, y + (long long)j0 * ldy, ldy,
+               c.N, nb);
+  }
+  return cudaGetLastError() == cudaSuccess ? FIO_OK : FIO_ECUDA;
 }
 
 inline double2 cdiv(double2 a, double2 b) {
@@ -223,6 +252,10 @@ inline double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 // G-dot x (which = 2); x, y FP64 with ld = N
 int precond(Ctx& c, Work& w, int which, const double2* x, double2* y, int prec) {
   if (prec == FIO_P64) return fio_apply_internal(c.op, which, x, y, c.N, c.b, FIO_P64, c.s);
+  // split-TF32 corrections run in FP32: closer to the factors' product (7e-7 against 2.6e-5 on the 2D
+  // n = 256 shapes), and since its large stages are on the tensor cores too, faster (2D n = 128, b = 32:
+  // 0.33 ms an apply against 0.45; n = 256 2.4 against 3.2)
+  if (prec == FIO_PTF32X3) prec = FIO_P32;
   const long long n = c.N * c.b;
   pdl_launch(true, k_to32, nblocks(n), 256, 0, c.s, x, w.v32[0], n);
   int rc = fio_apply_internal(c.op, which, w.v32[0], w.v32[1], c.N, c.b, prec, c.s);
@@ -258,6 +291,11 @@ void fio_solver_free(fio_op op) {
     op->solver = nullptr;
     op->solver_bytes = 0;
   }
+  if (op && op->solver_host) {
+    cudaFreeHost(op->solver_host);
+    op->solver_host = nullptr;
+    op->solver_host_bytes = 0;
+  }
 }
 
 extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b, int dtype,
@@ -284,21 +322,26 @@ extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b,
   Work w;
   int rc = get_work(op, b, restart, &w);
   if (rc) return rc;
-  Ctx c{op, rop, op->N, b, s, w.sc};
+  Ctx c{op, rop, op->N, b, s, w.host};
   c.outer = opts->outer;
   const double2* u = (const double2*)uv;
   double2* f = (double2*)fv;
   const long long N = op->N;
   std::vector<double2> tmp;
-  rc = dots(c, u, N, u, N, w.sc + 2 * b, &tmp);
+  c.host = w.host + b;
+  rc = dots(c, u, N, u, N, w.sc + 2 * b, nullptr);  // read with the next ones
+  c.host = w.host;
   if (rc) return rc;
+  std::vector<double2> fdot;
+  rc = opts->method != FIO_DIRECT ? dots(c, f, N, f, N, w.sc + 2 * b, &fdot)
+                                  : (cudaStreamSynchronize(s) == cudaSuccess ? FIO_OK : FIO_ECUDA);
+  if (rc) return rc;
+  tmp.assign(w.host + b, w.host + 2 * b);
   std::vector<double> unorm(b);
   for (int j = 0; j < b; ++j) unorm[j] = sqrt(tmp[j].x) > 0 ? sqrt(tmp[j].x) : 1.0;
   if (opts->method != FIO_DIRECT) {  // a zero initial guess needs no apply for its residual
-    rc = dots(c, f, N, f, N, w.sc + 2 * b, &tmp);
-    if (rc) return rc;
     c.f_zero = true;
-    for (int j = 0; j < b; ++j) c.f_zero = c.f_zero && tmp[j].x == 0.0;
+    for (int j = 0; j < b; ++j) c.f_zero = c.f_zero && fdot[j].x == 0.0;
   }
   std::vector<double> relres(b, 1.0);
   std::vector<int> iters(b, 0);
@@ -432,16 +475,16 @@ extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b,
         rc = fio_apply_internal(op, 0, Zt, Wv, N, b, FIO_P64, s);
         if (rc) return rc;
         std::vector<double2> h1((size_t)(k + 1) * b), h2((size_t)(k + 1) * b);
+        double2* hb = w.host + 2 * (size_t)b;  // behind the dots' scalars
         for (int pass = 0; pass < 2; ++pass) {
           dim3 grid(k + 1, b);
-          pdl_launch(true, k_basisdot, grid, kRedThreads, 0, s, V, vs, Wv, N, b, k + 1, w.Hd);
+          pdl_launch(true, k_basisdot, grid, kRedThreads, 0, s, V, vs, Wv, N, b, k + 1, w.Hd, hb + (size_t)pass * (k + 1) * b);
           pdl_launch(true, k_basis_sub, nblocks(N * b), 256, 0, s, V, vs, Wv, N, b, k + 1, w.Hd);
-          auto& dst = pass ? h2 : h1;
-          if (cudaMemcpyAsync(dst.data(), w.Hd, (size_t)(k + 1) * b * sizeof(double2), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-            return FIO_ECUDA;
         }
         rc = dots(c, Wv, N, Wv, N, w.sc + 2 * b, &tmp);
         if (rc) return rc;
+        h1.assign(hb, hb + h1.size());
+        h2.assign(hb + h1.size(), hb + 2 * h1.size());
         ++total_it;
         std::vector<double2> inv2(b);
         for (int j = 0; j < b; ++j) {
@@ -530,8 +573,9 @@ extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b,
       if (relres[j] <= tol) done[j] = 1;
     }
   }
-  if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) return FIO_ECUDA;
-  if (fio_tc_timeout_reset() > 0) return FIO_ETIMEOUT;
+  const int to = fio_sync_flag(op, s);
+  if (to < 0 || cudaGetLastError() != cudaSuccess) return FIO_ECUDA;
+  if (to > 0) return FIO_ETIMEOUT;
   bool conv = true;
   for (int j = 0; j < b; ++j) {
     const bool ok = relres[j] <= tol || opts->method == FIO_DIRECT;
