@@ -443,7 +443,7 @@ extern "C" const char* fio_strerror(int status) {
 // scratch pool: 5 work arrays of max(max_len, N) x b complex elements each
 // ---------------------------------------------------------------------------------------------
 int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void** fxbuf, size_t* fxbytes) {
-  const size_t per = (size_t)op->max_len * (size_t)b * elem;
+  const size_t per = (size_t)op->max_len * (size_t)(elem == 8 ? (b + 1) & ~1 : b) * elem;  // row_stride
   const size_t per_al = (per + 255) & ~(size_t)255;
   const size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
   const size_t need = 5 * per_al + fxneed;
@@ -483,6 +483,12 @@ thread_local Marks* g_marks = nullptr;
 inline void mark(cudaStream_t s) {
   if (g_marks) g_marks->mark(s);
 }
+
+// Row stride of the work vectors: in complex64 rounded up to even from b = 5 on, so that every row is
+// 16-byte aligned and the pipelined kernels serve odd counts too (they may read, never write, the odd
+// column; b = 13 at N = 4096: 0.36 ms a direct solve unpadded, 0.24 padded)
+template <typename V>
+inline int row_stride(int b) { return sizeof(V) == 8 && b >= 5 ? (b + 1) & ~1 : b; }
 
 template <typename V> const V* stage_M(const Stage& st);
 template <> const double2* stage_M<double2>(const Stage& st) { return st.M64; }
@@ -626,7 +632,7 @@ bool launch_small(const StageArgs<V>& a, cudaStream_t s) {
 template <typename V>
 bool pipe_ok(const StageArgs<V>& a) {
   const int vpc = 16 / (int)sizeof(V);
-  return a.xcs == 1 && a.xrs == a.b && a.C % vpc == 0 && a.b % vpc == 0 &&
+  return a.xcs == 1 && a.xrs >= a.b && a.xrs % vpc == 0 && a.C % vpc == 0 &&
          ((uintptr_t)a.M & 15) == 0 && ((uintptr_t)a.x & 15) == 0;
 }
 
@@ -746,7 +752,14 @@ bool variant_applies(const StageArgs<V>& a, int var) {
 template <typename V, bool ADJ>
 void launch_stage_dir(const StageArgs<V>& a, cudaStream_t s, int var) {
   if (var > 0 && launch_variant<V, ADJ>(a, s, var)) return;
+  // many blocks of at most 16 x 16: a warp each (a 64-row tile leaves three quarters of its rows
+  // idle); the same sums.  FP32 at b = 32: 4096 blocks 56 us in tiles, 18 so; 1024 blocks 20 and 12; 256
+  // blocks 12 and 10; 28 x 28 blocks, up to 512 of them, 8 to 10 us in tiles, 14 to 18 so
+  if (a.b >= 5 && a.xcs == 1 && a.R <= 16 && a.C <= 16 && a.nblk >= 1024 && launch_small<V, ADJ>(a, s)) return;
   if (a.b >= 5 && pipe_ok(a)) {
+    // complex64 from 17 right-hand sides on: contiguous thread tiles (variant 9; 252 x 252 blocks,
+    // b = 32: 0.109 ms a K-dot of 4 stages against 0.119), the same sums
+    if (a.b > 16 && launch_vt_if<V, ADJ, 16, 2, 8, 128>(a, s)) return;
     if (a.b <= 8) launch_pipe<V, ADJ, 8, 1, 2>(a, s);
     else if (a.b <= 16) launch_pipe<V, ADJ, 16, 1, 4>(a, s);
     else launch_pipe<V, ADJ, 16, 2, 4>(a, s);
@@ -1067,15 +1080,15 @@ void launch_stage(const Stage& st, bool adj, const V* x, long long xrs, long lon
 // levels have few, large blocks), partial sums into P, then k_partial_reduce adds the slices in a
 // fixed order straight into W (the stage's copy-back).  False when it does not apply.
 template <typename V>
-bool inplace_split(const Stage&, bool, V*, V*, long long, int, cudaStream_t) {
+bool inplace_split(const Stage&, bool, V*, V*, long long, int, int, cudaStream_t) {
   return false;
 }
 constexpr int kFp32SplitVariant = 12;
 
 // the FP32 CUDA-core split (variant 12): 128-row tiles of 8 x 4 thread tiles, about two CTAs per
 // SM slot, at least four 16-column chunks per slice
-bool inplace_split_fp32(const Stage& st, bool adj, float2* W, float2* P, long long pcap, int b, cudaStream_t s) {
-  StageArgs<float2> a = stage_args<float2>(st, adj, W, b, 1, W, b, 1, b);
+bool inplace_split_fp32(const Stage& st, bool adj, float2* W, float2* P, long long pcap, int b, int rs, cudaStream_t s) {
+  StageArgs<float2> a = stage_args<float2>(st, adj, W, rs, 1, W, rs, 1, b);
   if (!pipe_ok(a) || !a.tiles128 || a.ntiles128 <= 0) return false;
   const long long prow = (long long)st.nblk * (adj ? st.C : st.R);
   if (prow <= 0 || prow > pcap) return false;
@@ -1091,18 +1104,32 @@ bool inplace_split_fp32(const Stage& st, bool adj, float2* W, float2* P, long lo
   const bool ok = adj ? launch_vt<true, 8, 4, 8, 128, 16>(a, s) : launch_vt<false, 8, 4, 8, 128, 16>(a, s);
   if (!ok) return false;
   const long long tot = prow * b;
-  pdl_launch(true, k_partial_reduce, (unsigned)((tot + 255) / 256), 256, 0, s, P, a.ksplit, prow, b, st.out, W);
+  pdl_launch(true, k_partial_reduce, (unsigned)((tot + 255) / 256), 256, 0, s, P, a.ksplit, prow, b, st.out, W, rs);
   return true;
 }
 
+// Untuned, the split is the choice for the few large blocks of an operator above 4096 unknowns (the
+// root and the top HIF levels): fewer 128-row tiles than a third of the SMs (2D n = 128, the root of
+// 1346 rows at b = 32: FP32 0.125 ms whole, 0.035 split; split TF32 0.225 whole, 0.041 split; 64
+// blocks of 390 rows keep the whole form, 0.067 against 0.083).
+bool split_by_default(const Stage& st, bool adj, int b) {
+  const int tiles = adj ? st.n128_adj : st.n128_fwd;
+  return st.in_len > 4096 && b >= 17 && (long long)tiles * ((b + 31) / 32) * 3 < num_sms() &&
+         std::max(st.maxcols[0], st.maxcols[1]) >= 128;
+}
+
 template <>
-bool inplace_split<float2>(const Stage& st, bool adj, float2* W, float2* P, long long pcap, int b, cudaStream_t s) {
+bool inplace_split<float2>(const Stage& st, bool adj, float2* W, float2* P, long long pcap, int b, int rs, cudaStream_t s) {
   if (!P) return false;
   const int bk = rhs_bucket(b), dir = adj ? 1 : 0;
   const bool tc = use_tc<float2>(st, b, adj);
-  if (!tc || st.var[2 + g_tc_mode][dir][bk] == kFp32CoresVariant)
-    return st.var[1][dir][bk] == kFp32SplitVariant && inplace_split_fp32(st, adj, W, P, pcap, b, s);
-  if (st.var[2 + g_tc_mode][dir][bk] != kTmaSplitVariant) return false;
+  const bool dflt = split_by_default(st, adj, b);
+  if (!tc || st.var[2 + g_tc_mode][dir][bk] == kFp32CoresVariant) {
+    const int v = st.var[1][dir][bk];
+    return (v == kFp32SplitVariant || (v == 0 && dflt)) && inplace_split_fp32(st, adj, W, P, pcap, b, rs, s);
+  }
+  const int v = st.var[2 + g_tc_mode][dir][bk];
+  if (v != kTmaSplitVariant && !(v == 0 && dflt)) return false;
   const long long prow = (long long)st.nblk * (adj ? st.C : st.R);
   const int units = st.nunits[dir][0];
   if (prow <= 0 || units <= 0 || prow > pcap) return false;
@@ -1113,9 +1140,9 @@ bool inplace_split<float2>(const Stage& st, bool adj, float2* W, float2* P, long
   ks = std::min<long long>(ks, std::max(1, nch / 4));
   ks = (int)std::min<long long>(ks, pcap / prow);
   ks = std::max(1, std::min(ks, 64));
-  if (!launch_tma(st, adj, W, b, 1, nullptr, 0, 0, b, s, kTmaVariant, ks, P, 0)) return false;
+  if (!launch_tma(st, adj, W, rs, 1, nullptr, 0, 0, b, s, kTmaVariant, ks, P, 0)) return false;
   const long long tot = prow * b;
-  pdl_launch(true, k_partial_reduce, (unsigned)((tot + 255) / 256), 256, 0, s, P, ks, prow, b, st.out, W);
+  pdl_launch(true, k_partial_reduce, (unsigned)((tot + 255) / 256), 256, 0, s, P, ks, prow, b, st.out, W, rs);
   return true;
 }
 
@@ -1129,61 +1156,61 @@ constexpr int kDirectRows = kTileRows;
 // one INPLACE stage on the row-major work vector W (scratch S has the same shape; P, when not
 // null, is free scratch of pcap rows for the split variant)
 template <typename V>
-void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, cudaStream_t s, V* P = nullptr,
+void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, int rs, cudaStream_t s, V* P = nullptr,
                    long long pcap = 0) {
   if (st.nblk == 0) return;
-  if (inplace_split<V>(st, adj, W, P, pcap, b, s)) {
+  if (inplace_split<V>(st, adj, W, P, pcap, b, rs, s)) {
     mark(s);
     return;
   }
   // the fixed-point kernel reads W in a launch of its own (the gather), so it may write W
   const int var = st.var[type_index<V>()][adj ? 1 : 0][rhs_bucket(b)];
-  if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, W, b, 1, W, b, 1, b, s, var == kFxVariant)) {
+  if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, W, rs, 1, W, rs, 1, b, s, var == kFxVariant)) {
     mark(s);
     return;
   }
   const bool direct = std::max(st.maxcols[0], st.maxcols[1]) <= kDirectRows;
-  launch_stage<V>(st, adj, W, b, 1, direct ? W : S, b, 1, b, s);
+  launch_stage<V>(st, adj, W, rs, 1, direct ? W : S, rs, 1, b, s);
   if (!direct) {
     const long long nidx = (long long)st.nblk * st.R;
     const long long tot = nidx * b;
-    pdl_launch(true, k_scatter_back<V>, (unsigned)((tot + 255) / 256), 256, 0, s, st.out, nidx, S, W, b);
+    pdl_launch(true, k_scatter_back<V>, (unsigned)((tot + 255) / 256), 256, 0, s, st.out, nidx, S, W, b, rs);
   }
   mark(s);
 }
 
 template <typename V>
-void to_row(const V* X, long long ld, V* W, long long N, int b, cudaStream_t s) {
+void to_row(const V* X, long long ld, V* W, long long N, int b, int rs, cudaStream_t s) {
   dim3 grid((unsigned)((N + 31) / 32), (unsigned)((b + 31) / 32));
-  pdl_launch(true, k_col_to_row<V>, grid, dim3(32, 8), 0, s, X, ld, W, N, b);
+  pdl_launch(true, k_col_to_row<V>, grid, dim3(32, 8), 0, s, X, ld, W, N, b, rs);
   mark(s);
 }
 template <typename V>
-void to_col(const V* W, V* Y, long long ld, long long N, int b, cudaStream_t s) {
+void to_col(const V* W, V* Y, long long ld, long long N, int b, int rs, cudaStream_t s) {
   dim3 grid((unsigned)((N + 31) / 32), (unsigned)((b + 31) / 32));
-  pdl_launch(true, k_row_to_col<V>, grid, dim3(32, 8), 0, s, W, Y, ld, N, b);
+  pdl_launch(true, k_row_to_col<V>, grid, dim3(32, 8), 0, s, W, Y, ld, N, b, rs);
   mark(s);
 }
 
 // K-dot (adj = false) or K-dot* (adj = true): x (xrs, xcs) -> y (yrs, ycs); A, B ping-pong
 template <typename V>
 void bf_chain(fio_op op, bool adj, const V* x, long long xrs, long long xcs, V* y, long long yrs,
-              long long ycs, int b, V* A, V* B, cudaStream_t s) {
+              long long ycs, int b, V* A, V* B, int rs, cudaStream_t s) {
   const int n = op->n_bf;
   const V* cur = x;
   long long crs = xrs, ccs = xcs;
   if (b >= 5 && xrs == 1 && n > 1) {
     // caller's column-major input -> row-major work array, so every stage streams whole rows
-    to_row<V>(x, xcs, B, op->N, b, s);
+    to_row<V>(x, xcs, B, op->N, b, rs, s);
     cur = B;
-    crs = b;
+    crs = rs;
     ccs = 1;
   }
   for (int k = 0; k < n; ++k) {
     const Stage& st = op->st[adj ? n - 1 - k : k];
     const bool last = k == n - 1;
     V* dst = last ? y : ((k & 1) ? B : A);
-    const long long drs = last ? yrs : b, dcs = last ? ycs : 1;
+    const long long drs = last ? yrs : rs, dcs = last ? ycs : 1;
     launch_stage<V>(st, adj, cur, crs, ccs, dst, drs, dcs, b, s);
     mark(s);
     cur = dst;
@@ -1195,12 +1222,12 @@ void bf_chain(fio_op op, bool adj, const V* x, long long xrs, long long xcs, V* 
 // G-dot on the row-major work vector W in place; S scratch; P (max_len rows) free scratch for the
 // split in-place stages
 template <typename V>
-void g_sweep(fio_op op, V* W, V* S, int b, cudaStream_t s, V* P = nullptr) {
+void g_sweep(fio_op op, V* W, V* S, int b, int rs, cudaStream_t s, V* P = nullptr) {
   const int h0 = op->n_bf, nh = op->n_hif;
   const long long pc = op->max_len;
-  for (int t = 0; t < nh; ++t) inplace_stage<V>(op->st[h0 + t], false, W, S, b, s, P, pc);
-  for (int t = 0; t < op->n_root; ++t) inplace_stage<V>(op->st[h0 + nh + t], false, W, S, b, s, P, pc);
-  for (int t = nh - 1; t >= 0; --t) inplace_stage<V>(op->st[h0 + t], true, W, S, b, s, P, pc);
+  for (int t = 0; t < nh; ++t) inplace_stage<V>(op->st[h0 + t], false, W, S, b, rs, s, P, pc);
+  for (int t = 0; t < op->n_root; ++t) inplace_stage<V>(op->st[h0 + nh + t], false, W, S, b, rs, s, P, pc);
+  for (int t = nh - 1; t >= 0; --t) inplace_stage<V>(op->st[h0 + t], true, W, S, b, rs, s, P, pc);
 }
 
 int check_args(fio_op op, const void* x, const void* y, int64_t ld, int b, int dtype, int prec) {
@@ -1232,18 +1259,19 @@ enum Which { W_K = 0, W_KADJ = 1, W_G = 2, W_INV = 3 };
 // the apply `w` from x to y (both column-major, leading dimension ld) with work arrays A, B, W
 template <typename V>
 void apply_core(fio_op op, Which w, const V* x, V* y, int64_t ld, int b, V* A, V* B, V* W, cudaStream_t s) {
+  const int rs = row_stride<V>(b);
   switch (w) {
-    case W_K: bf_chain<V>(op, false, x, 1, ld, y, 1, ld, b, A, B, s); break;
-    case W_KADJ: bf_chain<V>(op, true, x, 1, ld, y, 1, ld, b, A, B, s); break;
+    case W_K: bf_chain<V>(op, false, x, 1, ld, y, 1, ld, b, A, B, rs, s); break;
+    case W_KADJ: bf_chain<V>(op, true, x, 1, ld, y, 1, ld, b, A, B, rs, s); break;
     case W_G:
-      to_row<V>(x, ld, W, op->N, b, s);
-      g_sweep<V>(op, W, A, b, s, B);
-      to_col<V>(W, y, ld, op->N, b, s);
+      to_row<V>(x, ld, W, op->N, b, rs, s);
+      g_sweep<V>(op, W, A, b, rs, s, B);
+      to_col<V>(W, y, ld, op->N, b, rs, s);
       break;
     case W_INV:
-      bf_chain<V>(op, true, x, 1, ld, W, b, 1, b, A, B, s);
-      g_sweep<V>(op, W, A, b, s, B);
-      to_col<V>(W, y, ld, op->N, b, s);
+      bf_chain<V>(op, true, x, 1, ld, W, rs, 1, b, A, B, rs, s);
+      g_sweep<V>(op, W, A, b, rs, s, B);
+      to_col<V>(W, y, ld, op->N, b, rs, s);
       break;
   }
 }
@@ -1489,7 +1517,8 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
   int rc = fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn);
   if (rc) return rc;
   FxScratch fxs(fxb, fxn);
-  const size_t bytes = (size_t)op->max_len * b * sizeof(V);
+  const int rs = row_stride<V>(b);
+  const size_t bytes = (size_t)op->max_len * rs * sizeof(V);
   V* X = (V*)bufs[0];
   V* Y = (V*)bufs[1];
   if (cudaMemsetAsync(X, 0, bytes, s) != cudaSuccess || cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess)
@@ -1512,7 +1541,7 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
       const int ti = tc ? 2 + g_tc_mode : type_index<V>();
       int best = 0;
       if (st.nblk > 0) {
-        const StageArgs<V> a = stage_args<V>(st, adj, X, b, 1, Y, b, 1, b);
+        const StageArgs<V> a = stage_args<V>(st, adj, X, rs, 1, Y, rs, 1, b);
         float tbest = -1.f;
         const int ncand = tc ? 9 : kNCand + 1;
         for (int k = 0; k < ncand; ++k) {
@@ -1527,7 +1556,7 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
                 [&] {
                   if (!tc && var != kFxVariant && (!variant_applies<V>(a, var) || is_3m_variant(var))) return false;
                   st.var[ti][dir][bucket] = (int8_t)var;
-                  inplace_stage<V>(st, adj, X, Y, b, s, (V*)bufs[2], op->max_len);
+                  inplace_stage<V>(st, adj, X, Y, b, rs, s, (V*)bufs[2], op->max_len);
                   return true;
                 },
                 s, e0, e1);
@@ -1541,10 +1570,10 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
                 },
                 s, e0, e1);
           } else if (tc) {
-            t = time_launch([&] { return launch_tc(st, adj, (const float2*)X, b, 1, (float2*)Y, b, 1, b, s, var); },
+            t = time_launch([&] { return launch_tc(st, adj, (const float2*)X, rs, 1, (float2*)Y, rs, 1, b, s, var); },
                             s, e0, e1);
           } else if (var == kFxVariant) {
-            t = time_launch([&] { return launch_fx<V>(st, adj, X, b, 1, Y, b, 1, b, s, true); }, s, e0, e1);
+            t = time_launch([&] { return launch_fx<V>(st, adj, X, rs, 1, Y, rs, 1, b, s, true); }, s, e0, e1);
           } else if (adj) {
             t = time_launch([&] { return launch_variant<V, true>(a, s, var); }, s, e0, e1);
           } else {
@@ -1706,7 +1735,7 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
   };
   if (rc == FIO_OK) {
     const long long N = op->N;
-    to_row<double2>((const double2*)x, ld, W64, N, b, s);  // both chains start from the same values
+    to_row<double2>((const double2*)x, ld, W64, N, b, b, s);  // both chains start from the same values
     convert_in(W64, W, N * b, s);
     if (which != 2) {
       const bool adj = which != 0;
@@ -1730,8 +1759,8 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
     if (which >= 2) {
       const int h0 = op->n_bf, nh = op->n_hif;
       auto step = [&](const Stage& st, bool adj) {
-        inplace_stage<double2>(st, adj, W64, A64, b, s);
-        inplace_stage<V>(st, adj, W, A, b, s, B, op->max_len);
+        inplace_stage<double2>(st, adj, W64, A64, b, b, s);
+        inplace_stage<V>(st, adj, W, A, b, b, s, B, op->max_len);
         record(W64, W, N * b);
       };
       for (int t = 0; t < nh && rc == FIO_OK; ++t) step(op->st[h0 + t], false);
@@ -1819,11 +1848,11 @@ int noalloc_scratch(void** out, void** fx) {
 }
 
 template <typename V>
-void inv_with_buffers(fio_op op, const V* u, V* f, int64_t ld, int b, V* A, V* B, V* W,
+void inv_with_buffers(fio_op op, const V* u, V* f, int64_t ld, int b, int rs, V* A, V* B, V* W,
                       cudaStream_t s) {
-  bf_chain<V>(op, true, u, 1, ld, W, b, 1, b, A, B, s);
-  g_sweep<V>(op, W, A, b, s, B);
-  to_col<V>(W, f, ld, op->N, b, s);
+  bf_chain<V>(op, true, u, 1, ld, W, rs, 1, b, A, B, rs, s);
+  g_sweep<V>(op, W, A, b, rs, s, B);
+  to_col<V>(W, f, ld, op->N, b, rs, s);
 }
 }  // namespace
 
@@ -1835,8 +1864,11 @@ extern "C" int fio_apply_inv_noalloc(fio_op op, const void* u, void* f, int64_t 
   if (op->n_root == 0) return FIO_ENOTSUP;
   if (b == 0) return FIO_OK;
   const size_t es = precision == FIO_P64 ? sizeof(double2) : sizeof(float2);
-  const size_t per = (((size_t)op->max_len * (size_t)b * es) + 255) & ~(size_t)255;
-  if (per > FIO_NOALLOC_SCRATCH_BYTES / 3) return FIO_EINVAL;  // does not fit the static scratch
+  auto per_of = [&](int rs) { return (((size_t)op->max_len * (size_t)rs * es) + 255) & ~(size_t)255; };
+  if (per_of(b) > FIO_NOALLOC_SCRATCH_BYTES / 3) return FIO_EINVAL;  // does not fit the static scratch
+  int rs = precision == FIO_P64 ? row_stride<double2>(b) : row_stride<float2>(b);
+  if (per_of(rs) > FIO_NOALLOC_SCRATCH_BYTES / 3) rs = b;  // the padded rows do not: unpadded
+  const size_t per = per_of(rs);
   void *base = nullptr, *fxb = nullptr;
   rc = noalloc_scratch(&base, &fxb);
   if (rc) return rc;
@@ -1847,13 +1879,13 @@ extern "C" int fio_apply_inv_noalloc(fio_op op, const void* u, void* f, int64_t 
   // Nothing here needs clearing: every stage writes all of its outputs before a later stage
   // reads them, so contents left by an earlier call are never read.
   if (precision == FIO_P64) {
-    inv_with_buffers<double2>(op, (const double2*)u, (double2*)f, ld, b, (double2*)p,
+    inv_with_buffers<double2>(op, (const double2*)u, (double2*)f, ld, b, rs, (double2*)p,
                               (double2*)(p + per), (double2*)(p + 2 * per), s);
   } else {
     // the stage arithmetic of the complex64 path (FP32 CUDA cores or a tensor-core mode), as in
     // fio_apply_inv
     TcMode m(tc_mode_of(precision));
-    inv_with_buffers<float2>(op, (const float2*)u, (float2*)f, ld, b, (float2*)p,
+    inv_with_buffers<float2>(op, (const float2*)u, (float2*)f, ld, b, rs, (float2*)p,
                              (float2*)(p + per), (float2*)(p + 2 * per), s);
   }
   return finish(s);

@@ -17,12 +17,12 @@ using namespace fio;
 
 namespace {
 
-// Stages the kernel may take.  In operators of at most kSmallOp unknowns only those with at least
-// kMinUnits 128-row tiles: their small and in-place stages keep the CUDA-core sums, which every tile
-// shape reproduces bit for bit.  Above, FP64 takes every stage (a CUDA-core FP64 tile of a 28-row
-// block takes 55 us whatever the number of blocks; this kernel 8 us), FP32 those with kMinUnits
-// tiles whose blocks have more than kSmallDim rows or columns.
-constexpr int64_t kSmallOp = 4096;
+// Stages the kernel may take.  In FP64: all of an operator above kSmallOp unknowns; in smaller ones,
+// above kTinyOp, those with at least kMinUnits 128-row tiles or blocks of at most one 64-row tile (a
+// CUDA-core FP64 tile of a 28-row block takes 22 us at b = 8 and 55 at b = 32 whatever the number of
+// blocks; this kernel 8 to 12): the rest keeps the CUDA-core sums, which every tile shape reproduces bit
+// for bit.  In FP32: with kMinUnits tiles, blocks of more than kSmallDim rows or columns.
+constexpr int64_t kSmallOp = 4096, kTinyOp = 1024;
 constexpr int kMinUnits = 96;
 constexpr int kSmallDim = 32;
 
@@ -121,7 +121,8 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
     const bool few = std::min(n.x, n.y) < kMinUnits;
     Plan p;
     p.stage = (int)si;
-    p.want[0] = ok && want[0] && (op->N > kSmallOp || !few);
+    const bool narrow = std::max(st.maxcols[0], st.maxcols[1]) <= 64;
+    p.want[0] = ok && want[0] && (op->N > kSmallOp || !few || (op->N > kTinyOp && narrow));
     p.want[1] = ok && want[1] && !few && std::max(st.maxcols[0], st.maxcols[1]) > kSmallDim;
     if (!p.want[0] && !p.want[1]) continue;
     p.exps = nexp;
@@ -226,22 +227,31 @@ size_t fx_scratch_bytes(fio_op op, int b, size_t elem) {
   return al256((size_t)op->fx_max_cols[t] * (size_t)b * elem) + al256((size_t)op->fx_max_blk * (size_t)b * sizeof(int));
 }
 
-// The built-in choice.  FP64 from b = 5 on: the CUDA-core kernels need 4 to 20 times as long on every
-// stage.  FP64 at b <= 4 (k_stage_vec streams the factor at 0.8 TFLOP/s forward, 1.1 adjoint) and FP32
-// by estimated time: K steps of the busiest SM at the measured time a step, against the CUDA-core rate
-// (31 TFLOP/s up to 16 right-hand sides, 42 above).  Measured on both sides of the line: blocks of
-// 415 x 250 at FP32 b = 32 0.34 ms against 0.60, of 58 x 58 0.035 against 0.030; FP64 b = 1 58 x 58
-// adjoint 0.0319 against 0.0290, 415 x 250 0.38 against 0.75.  FP32 also needs two tiles for every SM:
-// below, the few tiles' own latency decides and the smaller CUDA-core tiles fill the chip better.
+// The built-in choice.  FP64 from b = 5 on: the CUDA-core kernels need 2 to 20 times as long on every
+// stage.  FP64 at b <= 4 and FP32 by estimated time, in microseconds.
+//   this kernel   9 for its two launches, and the busiest SM's K steps at their measured time, or
+//                 1.4 a unit (the drain of a short one)
+//   FP64, b <= 4  k_stage_vec: 7, and b times the entries a CTA slot streams, at 2.2 ns (wide blocks) to
+//                 4 ns (narrow ones) forward and 1.25 to 1.9 adjoint.  Measured on both sides of the line,
+//                 b = 1: 141 blocks of 58 x 58 forward 28 against 16, adjoint 15 against 16; 4096 blocks
+//                 of 16 x 16 adjoint 30 against 63; 72 blocks of 228 x 228 67 against 27
+//   FP32          31 TFLOP/s up to 16 right-hand sides, 42 above.  Measured at b = 32: blocks of 415 x 250
+//                 0.60 ms against 0.34, of 58 x 58 0.030 against 0.035.  FP32 also needs two tiles for
+//                 every SM: below, the smaller CUDA-core tiles fill the chip better.
 bool fx_takes(const Stage& st, bool adj, bool wide, int b) {
   if (!st.fx_ok[wide ? 0 : 1]) return false;
+  if (wide && b > 4) return true;
   const int sms = sm_count(), bt = wide ? (b <= 8 ? 8 : 16) : (b <= 8 ? 8 : b <= 16 ? 16 : 32);
   const long long nrt = (b + bt - 1) / bt, units = st.n_fx_units[adj] * nrt;
-  // microseconds: K steps of the busiest SM, against the CUDA-core kernels' rate
   const double step = wide ? (bt == 8 ? 0.55 : 0.80) : (bt == 8 ? 0.33 : bt == 16 ? 0.37 : 0.45);
-  const double waves = (double)((units + sms - 1) / sms) / ((double)units / sms);
-  const double fx = 4.0 + step * waves * (double)(st.fx_steps[adj] * nrt) / sms;
-  if (wide) return b > 4 || fx < 8e-6 * (double)st.nnz * b / (adj ? 1.1 : 0.8);
+  const double a_unit = std::max(1.4, step * (double)st.fx_steps[adj] / st.n_fx_units[adj]);
+  const double fx = 9.0 + a_unit * (double)((units + sms - 1) / sms);
+  if (wide) {
+    const bool broad = std::max(st.maxcols[0], st.maxcols[1]) >= 128;
+    const double ns = adj ? (broad ? 1.25 : 1.9) : (broad ? 2.2 : 4.0);
+    const int tiles = std::min(sms, std::max(1, adj ? st.ntiles_adj : st.ntiles_fwd));
+    return fx < 7.0 + 1e-3 * b * ns * (double)st.nnz / tiles;
+  }
   const int bp = b <= 16 ? 16 : (b + 31) / 32 * 32;
   return b > 8 && units >= 2LL * sms && fx < 8e-6 * (double)st.nnz * bp / (b <= 16 ? 31.0 : 42.0);
 }

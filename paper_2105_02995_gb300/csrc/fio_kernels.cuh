@@ -739,24 +739,36 @@ __global__ void __launch_bounds__(32 * kSmallWarps) k_stage_small(StageArgs<V> a
   const int* rowidx = ADJ ? a.in + (size_t)blk * a.C : a.out + (size_t)blk * a.R;
   const int* colidx = ADJ ? a.out + (size_t)blk * a.R : a.in + (size_t)blk * a.C;
   for (int e = lane; e < RC; e += 32) sm[e] = M[e];
-  pdl_wait();
+  // a lane keeps one entry of each index list (at most 32), so that no later load waits for one
+  const int ci = lane < ncols ? colidx[lane] : -1, ri = lane < nrows ? rowidx[lane] : -1;
   const int j = blockIdx.y * 32 + lane;
   const bool on = j < a.b;
-#pragma unroll 4
+  pdl_wait();
+#pragma unroll 8
   for (int c = 0; c < ncols; ++c) {
-    const int idx = colidx[c];
+    const int idx = __shfl_sync(0xffffffffu, ci, c);
     sx[c * 32 + lane] = (idx >= 0 && on) ? a.x[(long long)idx * a.xrs + (long long)j * a.xcs] : czero<V>();
   }
   __syncwarp();
-  for (int r = 0; r < nrows; ++r) {
-    const int oidx = rowidx[r];
-    if (oidx < 0) continue;
-    V acc = czero<V>();
+  for (int r0 = 0; r0 < nrows; r0 += 4) {  // four rows at a time: independent sums in flight
+    V acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = czero<V>();
+#pragma unroll 2
     for (int c = 0; c < ncols; ++c) {
-      const V m = ADJ ? sm[c * a.C + r] : sm[r * a.C + c];
-      acc = ADJ ? cmacc(acc, m, sx[c * 32 + lane]) : cmac(acc, m, sx[c * 32 + lane]);
+      const V xv = sx[c * 32 + lane];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int r = min(r0 + k, nrows - 1);
+        const V m = ADJ ? sm[c * a.C + r] : sm[r * a.C + c];
+        acc[k] = ADJ ? cmacc(acc[k], m, xv) : cmac(acc[k], m, xv);
+      }
     }
-    if (on) a.y[(long long)oidx * a.yrs + (long long)j * a.ycs] = acc;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int oidx = __shfl_sync(0xffffffffu, ri, min(r0 + k, 31));
+      if (r0 + k < nrows && oidx >= 0 && on) a.y[(long long)oidx * a.yrs + (long long)j * a.ycs] = acc[k];
+    }
   }
 }
 
@@ -889,7 +901,7 @@ __global__ void __launch_bounds__(256) k_stage_vec(StageArgs<V> a) {
 // rows back into the work vector W; blocks own disjoint rows, so no block reads a row another
 // block has already overwritten.
 template <typename V>
-__global__ void k_scatter_back(const int* idx, long long nidx, const V* S, V* W, int b) {
+__global__ void k_scatter_back(const int* idx, long long nidx, const V* S, V* W, int b, int rs) {
   pdl_go();
   pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -898,12 +910,12 @@ __global__ void k_scatter_back(const int* idx, long long nidx, const V* S, V* W,
   const int j = (int)(t - k * b);
   const int row = idx[k];
   if (row < 0) return;
-  W[(long long)row * b + j] = S[(long long)row * b + j];
+  W[(long long)row * rs + j] = S[(long long)row * rs + j];
 }
 
-// column-major (ld) <-> row-major (b) layout changes of an N x b array, 32 x 32 smem tiles
+// column-major (ld) <-> row-major (row stride rs) layout changes of an N x b array, 32 x 32 smem tiles
 template <typename V>
-__global__ void k_col_to_row(const V* X, long long ld, V* W, long long N, int b) {
+__global__ void k_col_to_row(const V* X, long long ld, V* W, long long N, int b, int rs) {
   pdl_go();
   pdl_wait();
   __shared__ V t[32][33];
@@ -918,12 +930,12 @@ __global__ void k_col_to_row(const V* X, long long ld, V* W, long long N, int b)
   for (int k = threadIdx.y; k < 32; k += blockDim.y) {
     const long long i = i0 + k;
     const int j = j0 + threadIdx.x;
-    if (i < N && j < b) W[i * b + j] = t[threadIdx.x][k];
+    if (i < N && j < b) W[i * rs + j] = t[threadIdx.x][k];
   }
 }
 
 template <typename V>
-__global__ void k_row_to_col(const V* W, V* Y, long long ld, long long N, int b) {
+__global__ void k_row_to_col(const V* W, V* Y, long long ld, long long N, int b, int rs) {
   pdl_go();
   pdl_wait();
   __shared__ V t[32][33];
@@ -932,7 +944,7 @@ __global__ void k_row_to_col(const V* W, V* Y, long long ld, long long N, int b)
   for (int k = threadIdx.y; k < 32; k += blockDim.y) {
     const long long i = i0 + k;
     const int j = j0 + threadIdx.x;
-    if (i < N && j < b) t[k][threadIdx.x] = W[i * b + j];
+    if (i < N && j < b) t[k][threadIdx.x] = W[i * rs + j];
   }
   __syncthreads();
   for (int k = threadIdx.y; k < 32; k += blockDim.y) {

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(tma::kThreads, 1) k_stage_tma(const TmaArgs a,
 // The slices of a split in-place stage summed in slice order, written into the work vector W at
 // the block rows' own indices (the in-place stage's copy-back): W[idx[r]][j] = sum_ks part[ks][r][j]
 // for every packed row r of the stage with idx[r] >= 0 (the blocks' index sets are disjoint).
-__global__ void k_partial_reduce(const float2* part, int ksplit, long long prow, int b, const int* idx, float2* W) {
+__global__ void k_partial_reduce(const float2* part, int ksplit, long long prow, int b, const int* idx, float2* W, int rs) {
   pdl_go();
   pdl_wait();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -532,7 +532,7 @@ __global__ void k_partial_reduce(const float2* part, int ksplit, long long prow,
     acc.x += v.x;
     acc.y += v.y;
   }
-  W[(long long)row * b + j] = acc;
+  W[(long long)row * rs + j] = acc;
 }
 
 }  // namespace fio
