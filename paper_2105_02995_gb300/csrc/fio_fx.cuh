@@ -108,6 +108,11 @@ static_assert(2 * kDrainRegs + 4 * kSliceRegs + kCtrlRegs <= 7 * 72, "more regis
 // chunks that a slicer group takes from one barrier are 8 apart, each consumed before the next is
 // issued, so that no group waits for a phase two ahead (which a parity wait would let pass).
 constexpr int kMaxRaw = 8;
+// Chunks that the copy warp asks L2 for ahead of the ring: shared memory holds three to five slots
+// beside the digit tiles, 55 KB in flight an SM, and under load HBM answers after 1.5 us or more.
+// (2D n = 256 FP64 b = 16: 3.23 ms without, 3.06 with; where several CTAs share a unit's factor they
+// already run ahead of one another, and 1D b = 64 lost 0.4%.)
+constexpr int kAhead = 6;
 constexpr uint32_t kBufCols = 256;
 constexpr int kPlain = 1 << 20;  // scale exponent that marks a column for plain()
 
@@ -161,6 +166,9 @@ __device__ __forceinline__ void bulk(uint32_t dst, const void* src, uint32_t byt
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst),
       "l"(src), "r"(bytes), "r"(tc::su32(bar)), "l"(policy)
       : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes, uint64_t policy) {
+  asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(src), "r"(bytes), "l"(policy) : "memory");
 }
 __device__ __forceinline__ void expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::su32(bar)), "r"(bytes) : "memory");
@@ -609,6 +617,25 @@ __global__ void __launch_bounds__(fx::kThreads, 1) k_stage_fx(const FxArgs a) {
       const uint64_t pol = evict_first();
       uint32_t ic = 0, s = 0, ph = 1;
       FxUnit nx = unit(blockIdx.x);
+      // the chunk to ask L2 for next: unit pu, pk chunks left of it
+      int pu = blockIdx.x, pk = 0;
+      uint32_t pbytes = 0;
+      const uint8_t* pA = nullptr;
+      auto ask = [&]() {
+        if (pk == 0) {
+          if (pu >= total) return;
+          const FxUnit f = unit(pu);
+          pu += gridDim.x;
+          pk = (f.ncols + KC - 1) / KC;
+          pbytes = (uint32_t)min(128, (f.nrows - f.r0 + 31) & ~31) * 128u;
+          pA = a.A + (size_t)(uint32_t)(W ? f.a64 : f.a32) * 128;
+        }
+        prefetch_l2(pA, pbytes, pol);
+        pA += pbytes;
+        --pk;
+      };
+      if (a.nrt == 1)
+        for (int q = 0; q < kAhead; ++q) ask();
       for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
         const FxUnit e = nx;
         nx = unit(u + gridDim.x);
@@ -622,6 +649,7 @@ __global__ void __launch_bounds__(fx::kThreads, 1) k_stage_fx(const FxArgs a) {
             ok = false;
             break;
           }
+          if (a.nrt == 1) ask();
           const uint32_t dst = base + OFF_RAW + s * RAW;
           uint64_t* full = &raw_full[ic % kMaxRaw];
           expect(full, abytes + xbytes);
