@@ -31,7 +31,9 @@
  * to the FP32 CUDA-core kernels.  The large stages of FIO_P64 and FIO_P32 run on the tensor cores in
  * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below their row's and column's largest,
  * digit products summed exactly, each output rounded once -- at least as close to the exact product
- * as the CUDA-core sums (columns with infinities, NaN or extreme exponents are summed plainly).
+ * as the CUDA-core sums (columns with infinities, NaN or extreme exponents are summed plainly).  The
+ * digit copies that this takes are made at upload where they fit half of the free device memory.
+ * fio_solve's corrections with inner = FIO_PTF32X3 run in FP32 (closer, and faster).
  * FIO_PDF takes complex128 vectors and applies a double-float copy
  * of the factors (each FP64 entry as an unevaluated sum of two floats, 48-bit significand) with
  * compensated (twice-working-precision) accumulation on the FP32 CUDA cores: FP64-class results

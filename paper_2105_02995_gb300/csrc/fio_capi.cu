@@ -445,8 +445,8 @@ extern "C" const char* fio_strerror(int status) {
 int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void** fxbuf, size_t* fxbytes) {
   const size_t per = (size_t)op->max_len * (size_t)(elem == 8 ? (b + 1) & ~1 : b) * elem;  // row_stride
   const size_t per_al = (per + 255) & ~(size_t)255;
-  const size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
-  const size_t need = 5 * per_al + fxneed;
+  size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
+  size_t need = 5 * per_al + fxneed;
   if (need > op->scratch_bytes) {
     if (op->scratch) {
       if (cudaStreamSynchronize(s) != cudaSuccess) return FIO_ECUDA;
@@ -454,8 +454,17 @@ int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void
       op->scratch = nullptr;
       op->scratch_bytes = 0;
     }
-    if (cudaMalloc(&op->scratch, need) != cudaSuccess) {
+    bool got = cudaMalloc(&op->scratch, need) == cudaSuccess;
+    if (!got && fxneed) {  // without the fixed-point kernel's part, from now on: the CUDA-core kernels serve
       cudaGetLastError();
+      fx_give_up(op, elem);
+      fxneed = 0;
+      need = 5 * per_al;
+      got = cudaMalloc(&op->scratch, need) == cudaSuccess;
+    }
+    if (!got) {
+      cudaGetLastError();
+      op->scratch = nullptr;
       return FIO_ENOMEM;
     }
     op->scratch_bytes = need;

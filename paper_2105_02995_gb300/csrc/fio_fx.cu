@@ -177,7 +177,11 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
   if (plans.empty()) return FIO_OK;
   const size_t oe = al256(units.size() * sizeof(FxUnit)), ox = oe + al256(nexp * sizeof(short)),
                ob = ox + al256(xofs.size() * sizeof(int2)), od = ob + al256(plans.size() * sizeof(int));
-  if (cudaMalloc(&op->fx, od + dbytes) != cudaSuccess) {  // no room for the copies: the CUDA-core kernels serve
+  // The copies take at most half of the free memory, so that scratch, solver vectors and other operators
+  // find the room they had without them; where they do not fit, the CUDA-core kernels serve.
+  size_t room = 0, all = 0;
+  if (cudaMemGetInfo(&room, &all) != cudaSuccess || od + dbytes > room / 2 ||
+      cudaMalloc(&op->fx, od + dbytes) != cudaSuccess) {
     cudaGetLastError();
     op->fx = nullptr;
     op->fx_max_cols[0] = op->fx_max_cols[1] = 0;
@@ -256,7 +260,10 @@ bool fx_takes(const Stage& st, bool adj, bool wide, int b) {
   return b > 8 && units >= 2LL * sms && fx < 8e-6 * (double)st.nnz * bp / (b <= 16 ? 31.0 : 42.0);
 }
 
+void fx_give_up(fio_op op, size_t elem) { op->fx_max_cols[elem == sizeof(double2) ? 0 : 1] = 0; }
+
 bool fx_all_wide(fio_op op) {
+  if (op->fx_max_cols[0] == 0) return false;
   for (const Stage& st : op->st)
     if (st.nblk && !st.fx_ok[0]) return false;
   return op->fx != nullptr;

@@ -151,6 +151,7 @@ inline bool is_tc_precision(int p) { return p == FIO_PTF32 || p == FIO_PBF16 || 
 // launch; the launch (false: not taken, nothing launched; *timeout is set by a bounded wait that gives up)
 int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>& mdims, cudaStream_t s);
 size_t fx_scratch_bytes(fio_op op, int b, size_t elem);
+void fx_give_up(fio_op op, size_t elem);  // no room for that scratch: the type's launches keep the other kernels
 bool fx_takes(const fio::Stage& st, bool adj, bool wide, int b);
 int fft_build(fio_op op, cudaStream_t s);  // the DFT's twiddle table (fio_fft.cu)
 bool fx_all_wide(fio_op op);  // every stage of the operator has an FP64 digit copy
