@@ -28,10 +28,9 @@
  * head and a TF32 tail and a product is summed as head*head + head*tail + tail*head (three MMAs
  * per step, FP32 accumulation; the dropped tail*tail term is ~2^-22 relative); same factors and
  * vectors as FIO_PTF32.  With fewer than 8 right-hand sides the tensor-core precisions fall back
- * to the FP32 CUDA-core kernels.  The large stages of FIO_P64 and FIO_P32 run on the tensor cores in
+ * to the FP32 CUDA-core kernels.  The large stages of FIO_P64 (and of FIO_P32 under variant 50) run on the tensor cores in
  * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below their row's and column's largest,
- * digit products summed exactly, each output rounded once -- at least as close to the exact product
- * as the CUDA-core sums (columns with infinities, NaN or extreme exponents are summed plainly).  The
+ * digit products summed exactly, each output rounded once (columns with infinities, NaN or extreme exponents are summed plainly).  The
  * digit copies that this takes are made at upload where they fit half of the free device memory.
  * fio_solve's corrections with inner = FIO_PTF32X3 run in FP32 (closer, and faster).
  * FIO_PDF takes complex128 vectors and applies a double-float copy

@@ -1020,6 +1020,7 @@ StageArgs<V> stage_args(const Stage& st, bool adj, const V* x, long long xrs, lo
 constexpr int kFxVariant = 50;
 thread_local void* g_fx_scratch = nullptr;
 thread_local size_t g_fx_bytes = 0;
+thread_local bool g_fx_corrections = false;  // within fio_apply_correction
 struct FxScratch {
   void* prev;
   size_t prev_bytes;
@@ -1037,6 +1038,10 @@ template <typename V>
 bool fx_rule(const Stage& st, bool adj, int b, bool pinned) {
   constexpr bool W = std::is_same<V, double2>::value;
   if (std::is_same<V, dfc>::value || !g_fx_scratch || (!W && g_tc_mode != 0)) return false;
+  // FP32 by the built-in rule in the solvers' split-TF32 corrections only: 30 bits below a row's and a
+  // column's largest are too few for the butterfly factors of a real operator (generalized Radon transform
+  // n = 256, b = 32, against the FP64 apply: 1.4e-6 on the CUDA cores, 7.7e-6 so, 2.4e-5 in split TF32)
+  if (!W && !pinned && !g_fx_corrections) return false;
   return st.fx_ok[W ? 0 : 1] && (pinned || fx_takes(st, adj, W, b));
 }
 // device address of the timeout flag (the kernel is in another translation unit), cached per device
@@ -1357,6 +1362,13 @@ int fio_tc_timeout_reset() {
   return v;
 }
 
+int fio_apply_correction(fio_op op, int which, const void* x, void* y, int64_t ld, int b, cudaStream_t s) {
+  g_fx_corrections = true;
+  const int rc = fio_apply_internal(op, which, x, y, ld, b, FIO_P32, s);
+  g_fx_corrections = false;
+  return rc;
+}
+
 int fio_sync_flag(fio_op op, cudaStream_t s) {
   if (!op->flag_host) {
     if (cudaMallocHost(&op->flag_host, sizeof(int)) != cudaSuccess) {
@@ -1556,7 +1568,7 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
         for (int k = 0; k < ncand; ++k) {
           const int var = tc ? kTcCand[k] : (k == kNCand ? kFxVariant : kCand[bucket][k]);
           if (var <= 0 && !tc) continue;
-          if (var == kFxVariant && !fx_rule<V>(st, adj, b, true)) continue;
+          if (var == kFxVariant && (ti == 1 || !fx_rule<V>(st, adj, b, true))) continue;
           float t;
           if (st.kind == 1) {
             // in-place stages: the whole stage (compute and copy-back, or split compute and

@@ -18,6 +18,9 @@
 //   hold them exactly whatever the order of summation.  Orders 0..S-1 are kept; what is dropped is
 //   about 2^-59 resp. 2^-27 of the product, below the rounding of an FMA chain of the operands'
 //   own type (FP64 chain 2^-51, FP32 2^-23 over 500 columns).
+//   That holds while a row's and a column's entries span few binary orders.  FP32's 6 spare bits are too
+//   few for the butterfly factors of a real operator (7.7e-6 against the FP64 apply, 1.4e-6 on the CUDA
+//   cores; generalized Radon transform n = 256), so FP32 serves corrections asked for in split TF32 only.
 //   The accumulators are drained every 128 / 256 columns into 96- resp. 64-bit integers, so a
 //   whole output is summed without any rounding and rounded once, to nearest, at the end.
 // Columns that hold infinities, NaN, or exponents near the end of the range are computed in plain

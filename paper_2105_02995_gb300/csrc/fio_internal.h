@@ -165,6 +165,9 @@ int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void
 // which: 0 K-dot, 1 K-dot*, 2 G-dot, 3 G-dot K-dot*; x, y column-major with leading dimension ld
 int fio_apply_internal(fio_op op, int which, const void* x, void* y, int64_t ld, int b, int prec,
                        cudaStream_t s);
+// the same in FP32 for a correction asked for in split TF32: large stages in 30-bit fixed point (closer than
+// split TF32, faster than the FP32 CUDA cores)
+int fio_apply_correction(fio_op op, int which, const void* x, void* y, int64_t ld, int b, cudaStream_t s);
 void fio_solver_free(fio_op op);
 // 1 when a tensor-core kernel's bounded wait gave up since the last call (and clear the flag),
 // 0 otherwise, -1 on a CUDA error

@@ -255,10 +255,11 @@ int precond(Ctx& c, Work& w, int which, const double2* x, double2* y, int prec) 
   // split-TF32 corrections run in FP32: closer to the factors' product (7e-7 against 2.6e-5 on the 2D
   // n = 256 shapes), and since its large stages are on the tensor cores too, faster (2D n = 128, b = 32:
   // 0.33 ms an apply against 0.45; n = 256 2.4 against 3.2)
-  if (prec == FIO_PTF32X3) prec = FIO_P32;
+  const bool split = prec == FIO_PTF32X3;
   const long long n = c.N * c.b;
   pdl_launch(true, k_to32, nblocks(n), 256, 0, c.s, x, w.v32[0], n);
-  int rc = fio_apply_internal(c.op, which, w.v32[0], w.v32[1], c.N, c.b, prec, c.s);
+  int rc = split ? fio_apply_correction(c.op, which, w.v32[0], w.v32[1], c.N, c.b, c.s)
+                 : fio_apply_internal(c.op, which, w.v32[0], w.v32[1], c.N, c.b, prec, c.s);
   if (rc) return rc;
   cudaMemsetAsync(y, 0, n * sizeof(double2), c.s);
   pdl_launch(true, k_add32, nblocks(n), 256, 0, c.s, w.v32[1], y, c.N, c.N, c.b);
