@@ -178,11 +178,13 @@ __device__ __forceinline__ void expect(uint64_t* bar, uint32_t bytes) {
 }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }  // -126 <= e <= 127
 
-// fixed-point value of a under the scale 2^E, as digits + 128
+// fixed-point value of a under the scale 2^E, as digits + 128 (zeros and subnormals have no implicit bit: with
+// it a zero would count as 2^-1023, up to 2^-41 of a column whose largest entry is near 2^-982)
 __device__ __forceinline__ uint2 fix(double a, int E) {
   const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
-  const int sh = min(max(1023 + E - (int)((hi >> 20) & 0x7ffu), 0), 63);
-  unsigned long long v = ((((unsigned long long)((hi & 0xfffffu) | 0x100000u)) << 32) | lo) << 10;
+  const uint32_t be = (hi >> 20) & 0x7ffu;
+  const int sh = min(max(1023 + E - (int)max(be, 1u), 0), 63);
+  unsigned long long v = ((((unsigned long long)((hi & 0xfffffu) | (be ? 0x100000u : 0u))) << 32) | lo) << 10;
   v >>= sh;
   const long long s = (long long)((int)hi >> 31);
   v = (v ^ (unsigned long long)s) - (unsigned long long)s + 0x8080808080808080ull;
