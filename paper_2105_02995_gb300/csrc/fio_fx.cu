@@ -32,7 +32,7 @@ template <typename R, bool ADJ>
 void pack(const Stage& st, const FxUnit* units, uint8_t* A, cudaStream_t s) {
   using V = typename fx::Cfg<R>::V;
   const V* M = (const V*)(std::is_same<R, double>::value ? (const void*)st.M64 : (const void*)st.M32);
-  k_fx_pack<R, ADJ><<<st.n_fx_units[ADJ], 256, 0, s>>>(units, M, ADJ ? st.in : st.out, ADJ ? st.out : st.in, st.fx_exp[ADJ],
+  k_fx_pack<R, ADJ><<<st.n_fx_units[ADJ], 256, 0, s>>>(units, M, ADJ ? st.in : st.out, ADJ ? st.out : st.in, st.fx_exp[ADJ], st.fx_cexp[ADJ],
                                                        (int)st.R, (int)st.C, A);
 }
 
@@ -126,7 +126,7 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
     p.want[1] = ok && want[1] && !few && std::max(st.maxcols[0], st.maxcols[1]) > kSmallDim;
     if (!p.want[0] && !p.want[1]) continue;
     p.exps = nexp;
-    nexp += (size_t)st.nblk * (st.R + st.C);
+    nexp += 2 * (size_t)st.nblk * (st.R + st.C);
     long long cols[2] = {0, 0};
     size_t bytes[2][2];
     const size_t u0 = units.size(), x0 = xofs.size();
@@ -197,11 +197,13 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
   for (size_t k = 0; k < plans.size(); ++k) {
     const Plan& p = plans[k];
     Stage& st = op->st[p.stage];
-    short* re = (short*)(p0 + oe) + p.exps;
-    st.fx_exp[0] = re;
-    st.fx_exp[1] = re + (size_t)st.nblk * st.R;
-    k_fx_exps<<<st.nblk, 512, 0, s>>>(st.M64, st.in, st.out, st.dims, (int)st.R, (int)st.C, re, re + (size_t)st.nblk * st.R,
-                                      bad + k);
+    short* ef = (short*)(p0 + oe) + p.exps;
+    short *er = ef + (size_t)st.nblk * st.C, *af = er + (size_t)st.nblk * st.R, *ar = af + (size_t)st.nblk * st.R;
+    st.fx_cexp[0] = ef;
+    st.fx_exp[0] = er;
+    st.fx_cexp[1] = af;
+    st.fx_exp[1] = ar;
+    k_fx_exps<<<st.nblk, 512, 0, s>>>(st.M64, st.in, st.out, st.dims, (int)st.R, (int)st.C, ef, er, af, ar, bad + k);
     for (int dir = 0; dir < 2; ++dir) {
       st.fx_units[dir] = (const FxUnit*)p0 + p.units[dir];
       st.fx_xofs[dir] = (const int2*)(p0 + ox) + p.xofs[dir];
@@ -284,6 +286,7 @@ bool fx_launch(const Stage& st, bool adj, bool wide, const void* x, long long xr
   a.X = (const uint8_t*)scratch;
   a.ej = (const int*)((uint8_t*)scratch + xb);
   a.rexp = st.fx_exp[dir];
+  a.cexp = st.fx_cexp[dir];
   a.rowidx = adj ? st.in : st.out;
   a.colidx = adj ? st.out : st.in;
   a.lrow = adj ? (int)st.C : (int)st.R;

@@ -7,20 +7,22 @@
 // FP16 ones with FP32 accumulation on the tensor cores.  The method is error-free splitting (Ozaki,
 // Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication", 2012) in its fixed-point form:
-//   a row r of the (complex, interleaved) factor is scaled by a power of two, 2^Er > max |a|, and a
-//   column j of the block's gathered vector entries by 2^ej > max |x|; each real becomes the
-//   integer v = a 2^(f-Er) (f = 62 in FP64, 30 in FP32: every entry down to 2^-9 resp. 2^-6 of its
-//   row's largest keeps all 53 resp. 24 bits), written in balanced base 256,
-//   v = sum_i d_i 256^(S-1-i), -128 <= d_i <= 127, S = 8 resp. 4 digits;
+//   the rows and columns of the (complex, interleaved) factor are scaled by powers of two, Er and Ec, to
+//   entries below 1 with one above 1/2 in every row (k_fx_exps); the column scales go into the
+//   gathered vector, whose entries are cut below 2^ej > max |x_c| 2^Ec; each real
+//   becomes an integer (f = 62 in FP64, 30 in FP32), v_a = a 2^(f-Er-Ec), v_x = x 2^(f+Ec-ej), written
+//   in balanced base 256, v = sum_i d_i 256^(S-1-i), -128 <= d_i <= 127, S = 8 resp. 4 digits;
 //   sum_k v_a v_x = sum_o 256^(2S-2-o) sum_{i+l=o} (D_i^a D_l^x): every digit product is an
 //   integer of at most 2^14, exact in FP16 x FP16 -> FP32, and sums of all products of one order o
 //   over at most 128 (FP64) or 256 (FP32) real columns stay within 2^24: the FP32 accumulators
 //   hold them exactly whatever the order of summation.  Orders 0..S-1 are kept; what is dropped is
 //   about 2^-59 resp. 2^-27 of the product, below the rounding of an FMA chain of the operands'
 //   own type (FP64 chain 2^-51, FP32 2^-23 over 500 columns).
-//   That holds while a row's and a column's entries span few binary orders.  FP32's 6 spare bits are too
-//   few for the butterfly factors of a real operator (7.7e-6 against the FP64 apply, 1.4e-6 on the CUDA
-//   cores; generalized Radon transform n = 256), so FP32 serves corrections asked for in split TF32 only.
+//   Those are errors of the largest scaled product of a block; an FMA chain's are of a row's own sum of
+//   products.  The column scales keep the two together: a real operator's HIF blocks have columns that
+//   differ by 2^6, and vectors that differ the other way.  Example 3 n = 128, G-dot in FP64 (relative
+//   error, CPU restatement): FMA chain 1.4e-15; rows scaled alone 1.6e-15, with columns 2.6e-16; right-hand
+//   sides that span 40 binary orders, n = 64: 1.1e-15, 1.5e-15, 3.6e-16; K-dot 1.6e-15, 1.2e-16, 1.2e-16.
 //   The accumulators are drained every 128 / 256 columns into 96- resp. 64-bit integers, so a
 //   whole output is summed without any rounding and rounded once, to nearest, at the end.
 // Columns that hold infinities, NaN, or exponents near the end of the range are computed in plain
@@ -80,6 +82,7 @@ struct FxArgs {
   const uint8_t* X;   // digit copy of the gathered vector (k_fx_gather)
   const int* ej;      // scale exponent of every (block, right-hand side), block stride b
   const short* rexp;  // scale exponent Er of every (block, row of the product), block stride lrow
+  const short* cexp;  // scale exponent Ec of every (block, column of the product), block stride lcol
   const int* rowidx;  // output index lists (forward: out, adjoint: in), block stride lrow
   const int* colidx;  // gather index lists, block stride lcol
   int lrow, lcol;
@@ -190,7 +193,10 @@ __device__ __forceinline__ uint2 fix(double a, int E) {
   v = (v ^ (unsigned long long)s) - (unsigned long long)s + 0x8080808080808080ull;
   return make_uint2((uint32_t)v, (uint32_t)(v >> 32));
 }
-__device__ __forceinline__ uint32_t fix(float a, int E) { return (uint32_t)__float2int_rn(a * pow2f(30 - E)) + 0x80808080u; }
+__device__ __forceinline__ uint32_t fix(float a, int E) {
+  const int s = 30 - E, h = s >> 1;  // -119 .. 176
+  return (uint32_t)__float2int_rn(a * pow2f(h) * pow2f(s - h)) + 0x80808080u;
+}
 template <typename F> __device__ __forceinline__ F fix_zero();
 template <> __device__ __forceinline__ uint2 fix_zero<uint2>() { return make_uint2(0x80808080u, 0x80808080u); }
 template <> __device__ __forceinline__ uint32_t fix_zero<uint32_t>() { return 0x80808080u; }
@@ -240,22 +246,30 @@ __device__ __noinline__ V plain(const V* M, int ldm, const int* cidx, int ncols,
   return acc;
 }
 
-// largest magnitude, as the upper word of its bits (and the lower words: FP64 subnormals)
-__device__ __forceinline__ uint32_t mag(double2 v) {
-  return max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
+// biased exponent of the larger part (subnormals: 1), -1 for zero
+__device__ __forceinline__ int biased(double2 v) {
+  const uint32_t x = (uint32_t)__double2hiint(v.x) & 0x7fffffffu, y = (uint32_t)__double2hiint(v.y) & 0x7fffffffu;
+  const uint32_t any = x | y | (uint32_t)__double2loint(v.x) | (uint32_t)__double2loint(v.y);
+  return any ? (int)max(max(x, y) >> 20, 1u) : -1;
 }
-__device__ __forceinline__ uint32_t mag(float2 v) {
-  return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
+__device__ __forceinline__ int biased(float2 v) {
+  const uint32_t m = max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
+  return m ? (int)max(m >> 23, 1u) : -1;
 }
-__device__ __forceinline__ uint32_t low_bits(double2 v) { return (uint32_t)(__double2loint(v.x) | __double2loint(v.y)); }
-__device__ __forceinline__ uint32_t low_bits(float2) { return 0u; }
 
-// scale exponent of a column from its largest magnitude (0 for a zero column)
+// An entry's exponent under its column scale, as a key > 0 that grows with it (0: zero); infinities and NaN above all
+constexpr int kKeyBias = 64, kKeyBad = 1 << 14;
+template <typename V>
+__device__ __forceinline__ int scale_key(V v, int ce) {
+  const int be = biased(v);
+  return be < 0 ? 0 : be == (sizeof(V) == 16 ? 2047 : 255) ? kKeyBad : be + ce + kKeyBias;
+}
+// scale exponent of a gathered vector from its largest key (0 for a zero vector)
 template <typename R>
-__device__ __forceinline__ int col_exp(uint32_t m, uint32_t low) {
+__device__ __forceinline__ int col_exp(int key) {
   constexpr bool W = std::is_same<R, double>::value;
-  const int be = (int)(m >> (W ? 20 : 23));
-  if (m == 0 && low == 0) return 0;
+  if (key == 0) return 0;
+  const int be = key - kKeyBias;
   if (be < 40 || be > (W ? 2047 - 40 : 255 - 40)) return kPlain;
   return be - (W ? 1022 : 126);
 }
@@ -323,38 +337,34 @@ __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, i
   using V = typename C::V;
   using F = typename C::F;
   constexpr bool W = std::is_same<R, double>::value;
-  __shared__ uint32_t s_mag[BT], s_low[BT];
+  __shared__ int s_key[BT];
   const int blk = blockIdx.x, rt = blockIdx.y;
   const int j0 = rt * BT, wt = min(BT, a.b - j0);
   const int2 d = a.dims[blk];
   const int ncols = ADJ ? d.x : d.y;
   const int* cidx = a.colidx + (size_t)blk * a.lcol;
+  const short* cexp = a.cexp + (size_t)blk * a.lcol;
   const V* x = (const V*)a.x;
   const int tid = threadIdx.x;
   pdl_go();
-  if (tid < BT) s_mag[tid] = s_low[tid] = 0u;
+  if (tid < BT) s_key[tid] = 0;
   __syncthreads();
   pdl_wait();
   // lanes along the right-hand sides (BT a power of two; those beyond wt idle)
   const int j = tid % BT, c0 = tid / BT;
   constexpr int CS = 256 / BT;
-  uint32_t m = 0, lo = 0;
+  int m = 0;
   if (j < wt) {
 #pragma unroll 4
     for (int c = c0; c < ncols; c += CS) {
-      const int idx = cidx[c];
-      if (idx >= 0) {
-        const V v = x[(long long)idx * a.xrs + (long long)(j0 + j) * a.xcs];
-        m = max(m, mag(v));
-        lo |= low_bits(v);
-      }
+      const int idx = cidx[c], ce = cexp[c];
+      if (idx >= 0) m = max(m, scale_key(x[(long long)idx * a.xrs + (long long)(j0 + j) * a.xcs], ce));
     }
-    atomicMax(&s_mag[j], m);
-    if (W) atomicOr(&s_low[j], lo);
+    atomicMax(&s_key[j], m);
   }
   __syncthreads();
   if (j >= wt) return;
-  const int e = col_exp<R>(s_mag[j], s_low[j]);
+  const int e = col_exp<R>(s_key[j]);
   if (c0 == 0) ej[(size_t)blk * a.b + j0 + j] = e;
   const int nk = C::KPC * ((ncols + 8 * C::KPC - 1) / (8 * C::KPC));
   const int2 xo = a.xofs[blk];
@@ -373,12 +383,12 @@ __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, i
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int c = 4 * q + i;
-      const int idx = c < ncols ? cidx[c] : -1;
+      const int idx = c < ncols ? cidx[c] : -1, ce = c < ncols ? cexp[c] : 0;
       re[i] = im[i] = fix_zero<F>();
       if (idx >= 0) {
         const V v = x[(long long)idx * a.xrs + (long long)(j0 + j) * a.xcs];
-        re[i] = fix(v.x, e);
-        im[i] = fix(v.y, e);
+        re[i] = fix(v.x, e - ce);
+        im[i] = fix(v.y, e - ce);
       }
     }
     uint4* o = out + ((size_t)(q >> 1) * C::S + (q & 1)) * wt + j;
@@ -721,43 +731,80 @@ __global__ void __launch_bounds__(fx::kThreads, 1) k_stage_fx(const FxArgs a) {
 }
 
 // ---- upload --------------------------------------------------------------------------------------
-// Scale exponents: rexp[blk R + r] with |M[r][c]| < 2^rexp over the block's columns that are read
-// (and cexp[blk C + c] over its rows); an exponent outside -60 .. 60, an infinity or NaN marks the
-// stage in bad[0] (its factor then keeps the CUDA-core kernels).
-__global__ void k_fx_exps(const double2* M, const int* in, const int* out, const int2* dims, int R, int C, short* rexp,
-                          short* cexp, int* bad) {
+// Scale exponents of a stage per direction: ef, er (forward: columns C a block, rows R), af, ar (adjoint:
+// columns R a block, rows C).  A column's is half way between its largest entry and its largest entry under
+// the rows' own scales, both below the block's (for a Hermitian positive definite block the square root of
+// the diagonal: in either extreme alone one of a real operator's HIF stages loses bits, see above); a row's is
+// its largest entry under the columns' scales.  A largest entry or a scale outside 2^-60 .. 2^60, an
+// infinity or NaN marks the stage in bad[0] (its factor then keeps the CUDA-core kernels).
+__global__ void k_fx_exps(const double2* M, const int* in, const int* out, const int2* dims, int R, int C, short* ef,
+                          short* er, short* af, short* ar, int* bad) {
   const int blk = blockIdx.x;
   const double2* Mb = M + (size_t)blk * R * C;
   const int2 d = dims[blk];
   const int* bi = in + (size_t)blk * C;
   const int* bo = out + (size_t)blk * R;
-  auto put = [&](short* dst, uint32_t m) {
-    const int E = (int)(m >> 20) - 1022;
-    if (m && (E < -60 || E > 60)) atomicExch(bad, 1);
-    *dst = (short)(m ? E : 0);
+  ef += (size_t)blk * C;
+  er += (size_t)blk * R;
+  af += (size_t)blk * R;
+  ar += (size_t)blk * C;
+  constexpr int kNone = -32768;  // no entry but zeros
+  __shared__ int s_top[4];       // largest of er, ef, af, ar after the first two passes
+  if (threadIdx.x < 4) s_top[threadIdx.x] = kNone;
+  __syncthreads();
+  auto expo = [&](int r, int c) {
+    const int be = bo[r] >= 0 && bi[c] >= 0 ? fx::biased(Mb[(size_t)r * C + c]) : -1;
+    return be < 0 ? kNone : be - 1022;
   };
-  // rows: a warp each
-  for (int r = threadIdx.x >> 5; r < d.x; r += blockDim.x >> 5) {
-    uint32_t m = 0;
-    for (int c = threadIdx.x & 31; c < d.y; c += 32)
-      if (bi[c] >= 0) m = max(m, fx::mag(Mb[(size_t)r * C + c]));
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) put(rexp + (size_t)blk * R + r, bo[r] >= 0 ? m : 0u);
-  }
-  // columns: a thread each
-  for (int c = threadIdx.x; c < d.y; c += blockDim.x) {
-    uint32_t m = 0;
-    for (int r = 0; r < d.x; ++r)
-      if (bo[r] >= 0) m = max(m, fx::mag(Mb[(size_t)r * C + c]));
-    put(cexp + (size_t)blk * C + c, bi[c] >= 0 ? m : 0u);
-  }
+  // rowto[r], colto[c]: the largest of a row and of a column, under colby resp. rowby (or as they are)
+  auto maxima = [&](const short* colby, short* rowto, const short* rowby, short* colto, int* top) {
+    auto put = [&](short* dst, int m, int* t) {
+      if (m != kNone && (m < (top && colby ? -120 : -60) || m > 60)) atomicExch(bad, 1);
+      if (t) atomicMax(t, m);
+      *dst = (short)(m == kNone ? kNone : min(max(m, -120), 60));
+    };
+    for (int r = threadIdx.x >> 5; r < d.x; r += blockDim.x >> 5) {  // a warp each
+      int m = kNone;
+      for (int c = threadIdx.x & 31; c < d.y; c += 32) {
+        const int e = expo(r, c);
+        if (e != kNone) m = max(m, colby ? e - colby[c] : e);
+      }
+      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if ((threadIdx.x & 31) == 0) put(rowto + r, m, top ? top : nullptr);
+    }
+    for (int c = threadIdx.x; c < d.y; c += blockDim.x) {  // a thread each
+      int m = kNone;
+      for (int r = 0; r < d.x; ++r) {
+        const int e = expo(r, c);
+        if (e != kNone) m = max(m, rowby ? e - rowby[r] : e);
+      }
+      put(colto + c, m, top ? top + 1 : nullptr);
+    }
+    __syncthreads();
+  };
+  maxima(nullptr, er, nullptr, ef, s_top);
+  maxima(ef, af, er, ar, s_top + 2);
+  auto half = [&](short* own, short other, int t0, int t1) {
+    const int m = *own == kNone ? 0 : (*own - t0 + other - t1) >> 1;
+    if (m < -60) atomicExch(bad, 1);
+    *own = (short)max(m, -60);
+  };
+  for (int r = threadIdx.x; r < d.x; r += blockDim.x) half(af + r, er[r], s_top[2], s_top[0]);
+  for (int c = threadIdx.x; c < d.y; c += blockDim.x) half(ef + c, ar[c], s_top[1], s_top[3]);
+  __syncthreads();
+  maxima(ef, er, af, ar, nullptr);
+  for (int r = threadIdx.x; r < d.x; r += blockDim.x)
+    if (er[r] == kNone) er[r] = 0;
+  for (int c = threadIdx.x; c < d.y; c += blockDim.x)
+    if (ar[c] == kNone) ar[c] = 0;
 }
 
 // Digit copy of a factor for one direction: a CTA per unit, a thread per (row, half K step).
 // Rows and columns outside the block, or that are not read or written, are zero.
 template <typename R, bool ADJ>
 __global__ void __launch_bounds__(256) k_fx_pack(const FxUnit* units, const typename fx::Cfg<R>::V* M, const int* rowidx,
-                                                 const int* colidx, const short* rexp, int Rr, int Cc, uint8_t* A) {
+                                                 const int* colidx, const short* rexp, const short* cexp, int Rr, int Cc,
+                                                 uint8_t* A) {
   using namespace fx;
   using C = Cfg<R>;
   using V = typename C::V;
@@ -780,8 +827,9 @@ __global__ void __launch_bounds__(256) k_fx_pack(const FxUnit* units, const type
       re[i] = im[i] = fix_zero<F>();
       if (row && c < e.ncols && colidx[(size_t)e.blk * lcol + c] >= 0) {
         const V v = ADJ ? Mb[(size_t)c * Cc + r] : Mb[(size_t)r * Cc + c];
-        re[i] = fix(v.x, E);
-        im[i] = fix(v.y, E);
+        const int Ec = cexp[(size_t)e.blk * lcol + c];
+        re[i] = fix(v.x, E + Ec);
+        im[i] = fix(v.y, E + Ec);
       }
     }
     uint4* o = out + ((size_t)(q >> 1) * C::S + (q & 1)) * rp + rl;

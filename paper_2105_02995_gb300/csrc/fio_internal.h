@@ -62,11 +62,11 @@ struct Stage {
   // first 128-row tile, tiles, 0), largest first
   const int4* units[2][3] = {};
   int nunits[2][3] = {};
-  // fixed-point kernel per [forward, adjoint]: scale exponents of the product's rows, work units,
+  // fixed-point kernel per [forward, adjoint]: scale exponents of the product's rows and columns, work units,
   // column offsets of the blocks in the gathered vector and its columns, and the digit copies of
   // the factor per [FP64, FP32][direction]; fx_ok: the copies exist and every exponent is in range
   bool fx_ok[2] = {};
-  const short* fx_exp[2] = {};
+  const short *fx_exp[2] = {}, *fx_cexp[2] = {};
   const FxUnit* fx_units[2] = {};
   int n_fx_units[2] = {};
   const int2* fx_xofs[2] = {};

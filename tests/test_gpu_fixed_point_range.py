@@ -72,3 +72,52 @@ def test_zeros_in_tiny_columns(k):
     for w, ref in REFS.items():
         y = getattr(op, "apply_" + w)(dev(x * 2.0 ** -k)).cpu().numpy() * 2.0 ** k
         assert rel(y, ref(P, x)) < TOL64, w
+
+
+def graded(rng, m):
+    """Rows and columns that span 20 binary orders each."""
+    return np.exp2(rng.uniform(-20, 0, (m, 1))) * even(rng, m) * np.exp2(rng.uniform(-20, 0, (1, m)))
+
+
+def hermitian(rng, m):
+    """A scaled positive definite block, as HIF and root blocks are: diagonal 2^-16 .. 1."""
+    e, d = even(rng, m), np.exp2(rng.uniform(-8, 0, m))
+    return d[:, None] * (np.eye(m) + 0.2 * (e + e.conj().T)) * d
+
+
+def wide(S, x, adjoint):
+    """A stage's product in extended precision."""
+    return (S.conj().T if adjoint else S).tocsr().astype(np.clongdouble) @ x.astype(np.clongdouble)
+
+
+BLOCKS = {"even": (even, near_identity), "graded": (graded, hermitian), "hermitian": (hermitian, graded)}
+
+
+@pytest.mark.parametrize("vector", ["gaussian", "40 orders", "against the factor", "half against"])
+@pytest.mark.parametrize("kind", list(BLOCKS))
+def test_error_no_larger_than_an_fma_chain(kind, vector):
+    """Factors and vectors whose entries span many binary orders, large entries of the one meeting small
+    ones of the other: no further from the product in extended precision than the CUDA-core sums."""
+    op, P, N = operator(kind, *BLOCKS[kind])
+    b = 6
+    rng = np.random.default_rng(41)
+    for w, S, adjoint in (("K", P.bf[0], False), ("Kadj", P.bf[2], True), ("G", P.hif[0], False)):
+        x = gaussian(rng, N, b)
+        cols = abs(S.conj().T if adjoint else S).max(axis=0).toarray().ravel()[:, None]
+        x = {"gaussian": x, "40 orders": x * np.exp2(rng.uniform(-40, 0, (N, 1))), "against the factor": x / cols,
+             "half against": x / np.sqrt(cols)}[vector]
+        chain = {"K": [(s, False) for s in P.bf], "Kadj": [(s, True) for s in reversed(P.bf)],
+                 "G": [(P.hif[0], False), (P.root[0], False), (P.hif[0], True)]}[w]
+        want = x
+        for s, a in chain:
+            want = wide(s, want, a)
+        xd, fn = dev(x), getattr(op, "apply_" + w)
+        y = fn(xd).cpu().numpy()
+        try:
+            op.set_variant(b, binding.FIO_P64, 1)
+            z = fn(xd).cpu().numpy()
+        finally:
+            op.set_variant(b, binding.FIO_P64, 0)
+        assert not np.array_equal(y, z)  # the two kernels
+        ey, ez = (float(np.sqrt((np.abs(v - want) ** 2).sum() / (np.abs(want) ** 2).sum())) for v in (y, z))
+        assert ey <= ez, (w, ey, ez)
