@@ -509,13 +509,33 @@ template <> struct ChunkK<double2> { static constexpr int v = 16; };
 template <> struct ChunkK<float2> { static constexpr int v = 32; };
 template <> struct ChunkK<dfc> { static constexpr int v = 16; };
 
-// Stage launches whose CTAs are light enough to be started early (pdl_launch): complex multiply-adds
-// of a CTA's tile.  A 64 x 58 tile of 8 right-hand sides (30,000) gains 2.3 us a launch, one of
-// 64 x 228 x 32 (467,000) loses 15.
+int num_sms();
+
+// Stage launches whose CTAs are light enough to be started early (pdl_launch), by the complex
+// multiply-adds of a CTA's tile and the grid.  Early CTAs, of more than one launch ahead, take the places
+// that are free when they come, and later run two on one multiprocessor while others idle: a loss of up
+// to a tile's time against a gain of 2 us a launch.  The limits follow the type's rate (FP64 2 lanes an SM and
+// clock, FP32 128) and how much of the chip the grid covers.  Measured, speed of a K-dot or inverse against
+// plain launches, with the limits of the columns:
+//   a grid of at most an eighth of the SMs never shares one: any tile up to 110000 (1D N = 256, FP64
+//     b = 8 1.19, FP32 b = 16 1.67)
+//   at most half of the SMs      110000         smaller
+//     FP32  1D N = 1024 b = 8    1.71           1.36 (30000)
+//     double-float               0.93           1.03 (30000)   Example 3 n = 32, b = 16
+//     FP64  40 tiles 64 x 230    0.46           1.05 (8000)    PCG, b = 5
+//   more                         110000         smaller
+//     FP32  1D N = 16384 b = 16  0.94           1.05 (30000)
+//     FP64  1D N = 4096 b = 1    0.65           1.18 (2500, 0.65 at 8000)   K-dot*
 constexpr long long kLightMacs = 110000;
 template <bool ADJ, typename V>
-bool light(const StageArgs<V>& a, int rows, int rhs) {
-  return (long long)rows * (ADJ ? a.R : a.C) * std::min(rhs, a.b) <= kLightMacs * a.ksplit;
+bool light(const StageArgs<V>& a, int rows, int rhs, const dim3& grid) {
+  const long long ctas = (long long)grid.x * grid.y * grid.z, sms = num_sms();
+  const bool many = 2 * ctas > sms;
+  const long long limit = 8 * ctas <= sms                    ? kLightMacs
+                          : sizeof(V) == sizeof(float2)      ? (many ? 34000 : kLightMacs)
+                          : std::is_same<V, dfc>::value      ? (many ? 30000 : 50000)
+                                                             : (many ? 2500 : 12000);
+  return (long long)rows * (ADJ ? a.R : a.C) * std::min(rhs, a.b) <= limit * a.ksplit;
 }
 
 template <typename V, bool ADJ, int TX, int TB, int TR>
@@ -527,7 +547,7 @@ void launch_mm(StageArgs<V> a, cudaStream_t s) {
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + BT - 1) / BT));
-  pdl_launch(light<ADJ>(a, RT, BT), k_stage_mm<V, ADJ, TX, TB, TR, ChunkK<V>::v>, grid, 256, 0, s, a);
+  pdl_launch(light<ADJ>(a, RT, BT, grid), k_stage_mm<V, ADJ, TX, TB, TR, ChunkK<V>::v>, grid, 256, 0, s, a);
 }
 
 // Dynamic shared memory above 48 KB is opted into per kernel and per device: remember, per (device,
@@ -564,7 +584,7 @@ void launch_pipe(StageArgs<V> a, cudaStream_t s) {
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + S::BT - 1) / S::BT));
-  pdl_launch(light<ADJ>(a, S::RT, S::BT), k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK>, grid, 256, S::SMEM, s, a);
+  pdl_launch(light<ADJ>(a, S::RT, S::BT, grid), k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK>, grid, 256, S::SMEM, s, a);
 }
 // the same tiles with three real products per complex product (FP64 and double-float only)
 template <typename V, bool ADJ, int TX, int TB, int TR>
@@ -579,7 +599,7 @@ bool launch_pipe3(StageArgs<V> a, cudaStream_t s) {
     const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
     if (ncta == 0) return true;
     dim3 grid((unsigned)ncta, (unsigned)((a.b + S::BT - 1) / S::BT));
-    pdl_launch(light<ADJ>(a, S::RT, S::BT), k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK, true>, grid, 256, smem, s, a);
+    pdl_launch(light<ADJ>(a, S::RT, S::BT, grid), k_stage_mm_pipe<V, ADJ, TX, TB, TR, CK, true>, grid, 256, smem, s, a);
     return true;
   } else {
     return false;
@@ -603,7 +623,7 @@ bool launch_vt(StageArgs<float2> a, cudaStream_t s) {
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return true;
   dim3 grid((unsigned)ncta, (unsigned)((a.b + S::BT - 1) / S::BT), (unsigned)a.ksplit);
-  pdl_launch(light<ADJ>(a, S::RT, S::BT), k_stage_mm_vt<ADJ, TX, TB, TR, NT, CK, MINB>, grid, NT, S::SMEM, s, a);
+  pdl_launch(light<ADJ>(a, S::RT, S::BT, grid), k_stage_mm_vt<ADJ, TX, TB, TR, NT, CK, MINB>, grid, NT, S::SMEM, s, a);
   return true;
 }
 template <typename V, bool ADJ, int TX, int TB, int TR, int NT, int CK = 32,
@@ -657,7 +677,7 @@ bool launch_vec_b(StageArgs<V> a, cudaStream_t s) {
   a.ntiles = (nrows + kTileRows - 1) / kTileRows;
   const long long ncta = a.tiles ? a.ntiles_list : (long long)a.nblk * a.ntiles;
   if (ncta == 0) return true;
-  pdl_launch(light<ADJ>(a, kTileRows, B), k_stage_vec<V, ADJ, B>, (unsigned)ncta, 256, (size_t)need, s, a);
+  pdl_launch(light<ADJ>(a, kTileRows, B, dim3((unsigned)ncta)), k_stage_vec<V, ADJ, B>, (unsigned)ncta, 256, (size_t)need, s, a);
   return true;
 }
 template <typename V, bool ADJ>
