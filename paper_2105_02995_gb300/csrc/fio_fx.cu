@@ -27,6 +27,7 @@ constexpr int kMinUnits = 96;
 constexpr int kSmallDim = 32;
 
 inline size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
+inline int list_stride(int lcol) { return (lcol + 15) & ~15; }  // whole FP32 chunks, 16-byte aligned
 
 template <typename R, bool ADJ>
 void pack(const Stage& st, const FxUnit* units, uint8_t* A, cudaStream_t s) {
@@ -80,7 +81,9 @@ bool launch(FxArgs a, uint8_t* X, int* ej, cudaStream_t s) {
   // multiprocessors that finish first (2D n = 256 FP64 b = 1, 440 K steps an SM: 2.04 ms without, 2.10 with;
   // 1D N = 16384 b = 5, 15 K steps: 414 us without, 360 with)
   const bool early = (long long)a.steps * a.nrt <= 300LL * sm_count();
-  pdl_launch(early, k_fx_gather<R, ADJ, BT>, dim3((unsigned)a.nblk, (unsigned)a.nrt), 256, 0, s, a, X, ej);
+  const int groups = (a.maxcols + 4 * (256 / BT) - 1) / (4 * (256 / BT));
+  auto gather = groups <= 1 ? k_fx_gather<R, ADJ, BT, 1> : groups <= 2 ? k_fx_gather<R, ADJ, BT, 2> : k_fx_gather<R, ADJ, BT, 4>;
+  pdl_launch(early, gather, dim3((unsigned)a.nblk, (unsigned)a.nrt), 256, 0, s, a, X, ej);
   pdl_launch(true, k_stage_fx<R, ADJ, BT>, (unsigned)std::min<long long>(total, sm_count()), fx::kThreads, need, s, a);
   return true;
 }
@@ -101,12 +104,12 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
   struct Plan {
     int stage;
     bool want[2];
-    size_t units[2], exps, xofs[2], digits[2][2];  // offsets: entries, entries, entries, bytes
+    size_t units[2], exps, xofs[2], list[2], digits[2][2];  // offsets: entries, entries, entries, entries, bytes
   };
   std::vector<Plan> plans;
   std::vector<FxUnit> units;
   std::vector<int2> xofs;
-  size_t nexp = 0, dbytes = 0;
+  size_t nexp = 0, nlist = 0, dbytes = 0;
   for (size_t si = 0; si < op->st.size(); ++si) {
     Stage& st = op->st[si];
     int2 n = make_int2(0, 0);
@@ -127,6 +130,10 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
     if (!p.want[0] && !p.want[1]) continue;
     p.exps = nexp;
     nexp += 2 * (size_t)st.nblk * (st.R + st.C);
+    for (int dir = 0; dir < 2; ++dir) {
+      p.list[dir] = nlist;
+      nlist += (size_t)st.nblk * list_stride(dir ? st.R : st.C);
+    }
     long long cols[2] = {0, 0};
     size_t bytes[2][2];
     const size_t u0 = units.size(), x0 = xofs.size();
@@ -176,7 +183,8 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
   }
   if (plans.empty()) return FIO_OK;
   const size_t oe = al256(units.size() * sizeof(FxUnit)), ox = oe + al256(nexp * sizeof(short)),
-               ob = ox + al256(xofs.size() * sizeof(int2)), od = ob + al256(plans.size() * sizeof(int));
+               ol = ox + al256(xofs.size() * sizeof(int2)), ob = ol + al256(nlist * sizeof(int2)),
+               od = ob + al256(plans.size() * sizeof(int));
   // The copies take at most half of the free memory, so that scratch, solver vectors and other operators
   // find the room they had without them; where they do not fit, the CUDA-core kernels serve.
   size_t room = 0, all = 0;
@@ -205,6 +213,10 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
     st.fx_exp[1] = ar;
     k_fx_exps<<<st.nblk, 512, 0, s>>>(st.M64, st.in, st.out, st.dims, (int)st.R, (int)st.C, ef, er, af, ar, bad + k);
     for (int dir = 0; dir < 2; ++dir) {
+      const int lcol = (int)(dir ? st.R : st.C);
+      int2* list = (int2*)(p0 + ol) + p.list[dir];
+      k_fx_list<<<st.nblk, 128, 0, s>>>(dir ? st.out : st.in, st.fx_cexp[dir], st.dims, dir == 1, lcol, list_stride(lcol), list);
+      st.fx_list[dir] = list;
       st.fx_units[dir] = (const FxUnit*)p0 + p.units[dir];
       st.fx_xofs[dir] = (const int2*)(p0 + ox) + p.xofs[dir];
       for (int t = 0; t < 2; ++t) st.fxA[t][dir] = p.want[t] ? p0 + od + p.digits[t][dir] : nullptr;
@@ -286,11 +298,13 @@ bool fx_launch(const Stage& st, bool adj, bool wide, const void* x, long long xr
   a.X = (const uint8_t*)scratch;
   a.ej = (const int*)((uint8_t*)scratch + xb);
   a.rexp = st.fx_exp[dir];
-  a.cexp = st.fx_cexp[dir];
   a.rowidx = adj ? st.in : st.out;
   a.colidx = adj ? st.out : st.in;
   a.lrow = adj ? (int)st.C : (int)st.R;
   a.lcol = adj ? (int)st.R : (int)st.C;
+  a.list = st.fx_list[dir];
+  a.llist = list_stride(a.lcol);
+  a.maxcols = (st.maxcols[dir] + 15) & ~15;
   a.dims = st.dims;
   a.xofs = st.fx_xofs[dir];
   a.xcols = cols;

@@ -82,10 +82,12 @@ struct FxArgs {
   const uint8_t* X;   // digit copy of the gathered vector (k_fx_gather)
   const int* ej;      // scale exponent of every (block, right-hand side), block stride b
   const short* rexp;  // scale exponent Er of every (block, row of the product), block stride lrow
-  const short* cexp;  // scale exponent Ec of every (block, column of the product), block stride lcol
+  const int2* list;   // per block and column of the product: the index gathered there (-1: none), its scale
+  int llist;          // exponent Ec; block stride, a multiple of 16 not below lcol
   const int* rowidx;  // output index lists (forward: out, adjoint: in), block stride lrow
   const int* colidx;  // gather index lists, block stride lcol
   int lrow, lcol;
+  int maxcols;        // columns of the widest block, whole chunks
   const int2* dims;   // per block (valid rows, valid columns) of the forward block
   const int2* xofs;   // per block: columns before it in X (FP64, FP32 chunking)
   long long xcols;    // columns of one right-hand-side tile of X
@@ -329,74 +331,120 @@ template <int I> using Int = std::integral_constant<int, I>;
 }  // namespace fx
 
 // The gathered vector of every block as digits (layout above), and its columns' scale exponents.
-// A CTA per (block, right-hand-side tile): one pass for the columns' maxima, one (from L2) to cut.
-template <typename R, bool ADJ, int BT>
+// A CTA per (block, right-hand-side tile), a thread for every CS-th group of four columns of one
+// right-hand side.  Bound by the latency of its two dependent loads, list and vector: the entries of
+// up to HOLD groups stay in registers between the maximum and the cut (blocks of at most 4 CS HOLD columns;
+// no more than a stage needs, for the registers), longer blocks load them twice.
+template <typename R, bool ADJ, int BT, int HOLD>
 __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, int* ej) {
   using namespace fx;
   using C = Cfg<R>;
   using V = typename C::V;
   using F = typename C::F;
   constexpr bool W = std::is_same<R, double>::value;
+  constexpr int CS = 256 / BT;
   __shared__ int s_key[BT];
   const int blk = blockIdx.x, rt = blockIdx.y;
   const int j0 = rt * BT, wt = min(BT, a.b - j0);
   const int2 d = a.dims[blk];
   const int ncols = ADJ ? d.x : d.y;
-  const int* cidx = a.colidx + (size_t)blk * a.lcol;
-  const short* cexp = a.cexp + (size_t)blk * a.lcol;
+  const int nk = C::KPC * ((ncols + 8 * C::KPC - 1) / (8 * C::KPC)), nq = 2 * nk;
+  const int4* list = reinterpret_cast<const int4*>(a.list + (size_t)blk * a.llist);  // two columns each
   const V* x = (const V*)a.x;
   const int tid = threadIdx.x;
   pdl_go();
   if (tid < BT) s_key[tid] = 0;
-  __syncthreads();
-  pdl_wait();
   // lanes along the right-hand sides (BT a power of two; those beyond wt idle)
   const int j = tid % BT, c0 = tid / BT;
-  constexpr int CS = 256 / BT;
-  int m = 0;
-  if (j < wt) {
-#pragma unroll 4
-    for (int c = c0; c < ncols; c += CS) {
-      const int idx = cidx[c], ce = cexp[c];
-      if (idx >= 0) m = max(m, scale_key(x[(long long)idx * a.xrs + (long long)(j0 + j) * a.xcs], ce));
+  const bool on = j < wt;
+  struct Four {
+    V v[4];
+    int ce[4];
+  };
+  auto get = [&](Four& f, const int4& p, const int4& q) {
+    const int idx[4] = {p.x, p.z, q.x, q.z};
+    f.ce[0] = p.y;
+    f.ce[1] = p.w;
+    f.ce[2] = q.y;
+    f.ce[3] = q.w;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      f.v[i] = on && idx[i] >= 0 ? x[(long long)idx[i] * a.xrs + (long long)(j0 + j) * a.xcs] : czero<V>();
+  };
+  auto key = [&](const Four& f, int m) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m = max(m, scale_key(f.v[i], f.ce[i]));
+    return m;
+  };
+  const bool hold = HOLD < 4 || nq <= HOLD * CS;  // HOLD 1 and 2 are launched for stages that fit
+  Four held[HOLD];
+  int4 lp[HOLD], lq[HOLD];
+  const int4 none = make_int4(-1, 0, -1, 0);
+  if (hold) {
+#pragma unroll
+    for (int k = 0; k < HOLD; ++k) {
+      const int q = c0 + k * CS;
+      lp[k] = q < nq ? list[2 * q] : none;
+      lq[k] = q < nq ? list[2 * q + 1] : none;
     }
-    atomicMax(&s_key[j], m);
   }
   __syncthreads();
-  if (j >= wt) return;
+  pdl_wait();
+  int m = 0;
+  if (hold) {
+#pragma unroll
+    for (int k = 0; k < HOLD; ++k) get(held[k], lp[k], lq[k]);
+#pragma unroll
+    for (int k = 0; k < HOLD; ++k) m = key(held[k], m);
+  } else {
+#pragma unroll 4
+    for (int q = c0; q < nq; q += CS) {
+      Four f;
+      get(f, list[2 * q], list[2 * q + 1]);
+      m = key(f, m);
+    }
+  }
+  if (on) atomicMax(&s_key[j], m);
+  __syncthreads();
+  if (!on) return;
   const int e = col_exp<R>(s_key[j]);
   if (c0 == 0) ej[(size_t)blk * a.b + j0 + j] = e;
-  const int nk = C::KPC * ((ncols + 8 * C::KPC - 1) / (8 * C::KPC));
   const int2 xo = a.xofs[blk];
   uint4* out = reinterpret_cast<uint4*>(X + ((long long)rt * BT * a.xcols + (long long)(W ? xo.x : xo.y) * wt) * sizeof(V));
-  if (e == kPlain) {  // for fx::plain, entry by entry; the products of these bytes are not used
-    constexpr int PER = 16 / (int)sizeof(V);
-    for (int c = c0; c < 8 * nk; c += CS) {
-      const int idx = c < ncols ? cidx[c] : -1;
-      V* item = reinterpret_cast<V*>(out + ((size_t)(c >> 3) * C::S + (c & 7) / PER) * wt + j);
-      item[c % PER] = idx >= 0 ? x[(long long)idx * a.xrs + (long long)(j0 + j) * a.xcs] : czero<V>();
+  auto put = [&](int q, const Four& f) {  // half q & 1 of K step q / 2
+    uint4* o = out + ((size_t)(q >> 1) * C::S + (q & 1)) * wt + j;
+    if (e == kPlain) {  // for fx::plain, entry by entry; the products of these bytes are not used
+      constexpr int PER = 16 / (int)sizeof(V);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        V* item = reinterpret_cast<V*>(out + ((size_t)(q >> 1) * C::S + (4 * (q & 1) + i) / PER) * wt + j);
+        item[i % PER] = f.v[i];
+      }
+      return;
     }
-    return;
-  }
-  for (int q = c0; q < 2 * nk; q += CS) {  // four columns: half q & 1 of K step q / 2
     F re[4], im[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int c = 4 * q + i;
-      const int idx = c < ncols ? cidx[c] : -1, ce = c < ncols ? cexp[c] : 0;
-      re[i] = im[i] = fix_zero<F>();
-      if (idx >= 0) {
-        const V v = x[(long long)idx * a.xrs + (long long)(j0 + j) * a.xcs];
-        re[i] = fix(v.x, e - ce);
-        im[i] = fix(v.y, e - ce);
-      }
+      re[i] = fix(f.v[i].x, e - f.ce[i]);
+      im[i] = fix(f.v[i].y, e - f.ce[i]);
     }
-    uint4* o = out + ((size_t)(q >> 1) * C::S + (q & 1)) * wt + j;
     o[0] = digit_pair<0>(re, im);
     o[2 * wt] = digit_pair<1>(re, im);
     if constexpr (W) {
       o[4 * wt] = digit_pair<2>(re, im);
       o[6 * wt] = digit_pair<3>(re, im);
+    }
+  };
+  if (hold) {
+#pragma unroll
+    for (int k = 0; k < HOLD; ++k)
+      if (c0 + k * CS < nq) put(c0 + k * CS, held[k]);
+  } else {
+#pragma unroll 2
+    for (int q = c0; q < nq; q += CS) {
+      Four f;
+      get(f, list[2 * q], list[2 * q + 1]);
+      put(q, f);
     }
   }
 }
@@ -797,6 +845,13 @@ __global__ void k_fx_exps(const double2* M, const int* in, const int* out, const
     if (er[r] == kNone) er[r] = 0;
   for (int c = threadIdx.x; c < d.y; c += blockDim.x)
     if (ar[c] == kNone) ar[c] = 0;
+}
+
+// Gather list of a stage for one direction (FxArgs::list): a CTA a block
+static __global__ void k_fx_list(const int* colidx, const short* cexp, const int2* dims, bool adj, int lcol, int llist, int2* list) {
+  const int blk = blockIdx.x, ncols = adj ? dims[blk].x : dims[blk].y;
+  for (int c = threadIdx.x; c < llist; c += blockDim.x)
+    list[(size_t)blk * llist + c] = c < ncols ? make_int2(colidx[(size_t)blk * lcol + c], cexp[(size_t)blk * lcol + c]) : make_int2(-1, 0);
 }
 
 // Digit copy of a factor for one direction: a CTA per unit, a thread per (row, half K step).

@@ -67,6 +67,7 @@ struct Stage {
   // the factor per [FP64, FP32][direction]; fx_ok: the copies exist and every exponent is in range
   bool fx_ok[2] = {};
   const short *fx_exp[2] = {}, *fx_cexp[2] = {};
+  const int2* fx_list[2] = {};  // rows gathered and their columns' scale exponents
   const FxUnit* fx_units[2] = {};
   int n_fx_units[2] = {};
   const int2* fx_xofs[2] = {};
