@@ -32,7 +32,7 @@
  * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below their row's and column's largest,
  * digit products summed exactly, each output rounded once (columns with infinities, NaN or extreme exponents are summed plainly).  The
  * digit copies that this takes are made at upload where they fit half of the free device memory.
- * fio_solve's corrections with inner = FIO_PTF32X3 run in FP32 (closer, and faster).
+ * fio_solve's corrections with inner = FIO_PTF32X3 take them too (see there).
  * FIO_PDF takes complex128 vectors and applies a double-float copy
  * of the factors (each FP64 entry as an unevaluated sum of two floats, 48-bit significand) with
  * compensated (twice-working-precision) accumulation on the FP32 CUDA cores: FP64-class results
@@ -180,7 +180,10 @@ int fio_apply_inv_host(fio_op op, const void* u_host, void* f_host, int64_t ld, 
  *   FIO_IR      iterative refinement: residual r = u - K-dot f on complex128 vectors in
  *               opts->outer precision (FP64 or double-float), correction G-dot K-dot* r in
  *               opts->inner precision, FP64 update f += d.
- * (FIO_PTF32X3 as the inner precision runs as FIO_P32: closer to the factors' product, and faster.)
+ * With FIO_PTF32X3 as the inner precision of an iterative method, stages with work enough for it run in
+ * 30-bit fixed point (closer to the factors' product than split TF32, and faster), whatever is tuned,
+ * unless fio_set_variant pinned a variant for FIO_PTF32X3; the others run what is tuned or pinned for
+ * FIO_PTF32X3, and as FIO_P32 (closer, and faster than the untuned split-TF32 kernel) where nothing is.
  * Every method computes its true residuals u - K-dot f in opts->outer precision (PCG and GMRES
  * run their Krylov products in FP64 whatever opts->outer is).  With opts->residual_op (FIO_IR,
  * FIO_DIRECT) those residuals, and hence tol and info->relres, refer to that operator's K-dot:

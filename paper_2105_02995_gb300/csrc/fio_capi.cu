@@ -1057,7 +1057,7 @@ struct FxScratch {
 template <typename V>
 bool fx_rule(const Stage& st, bool adj, int b, bool pinned) {
   constexpr bool W = std::is_same<V, double2>::value;
-  if (std::is_same<V, dfc>::value || !g_fx_scratch || (!W && g_tc_mode != 0)) return false;
+  if (std::is_same<V, dfc>::value || !g_fx_scratch || (!W && g_tc_mode != 0 && !g_fx_corrections)) return false;
   // FP32 by the built-in rule in the solvers' split-TF32 corrections only: 30 bits below a row's and a
   // column's largest are too few for the butterfly factors of a real operator (generalized Radon transform
   // n = 256, b = 32, against the FP64 apply: 1.4e-6 on the CUDA cores, 7.7e-6 so, 2.4e-5 in split TF32)
@@ -1089,11 +1089,27 @@ bool launch_fx(const Stage& st, bool adj, const V* x, long long xrs, long long x
                            flag, s);
 }
 
+// a stage of a correction that was asked for in split TF32 (fio_apply_correction)
+template <typename V>
+bool launch_correction(const Stage& st, bool adj, const V* x, long long xrs, long long xcs, V* y, long long yrs, long long ycs,
+                       int b, cudaStream_t s) {
+  return g_fx_corrections && std::is_same<V, float2>::value && !st.x3_pinned[rhs_bucket(b)] &&
+         launch_fx<V>(st, adj, x, xrs, xcs, y, yrs, ycs, b, s, false);
+}
+
+// Whether the tensor-core precision's own kernels run a stage.  In a correction not where nothing is tuned or
+// pinned for split TF32: the FP32 CUDA cores are closer there, and faster than the untuned split-TF32 kernel
+// (refinement 2D n = 128: b = 32 5.0 ms against 5.5, b = 8 3.3 against 4.8; tuned split TF32 4.8 and 2.9).
+template <typename V>
+bool tc_serves(const Stage& st, int b, bool adj) {
+  return use_tc<V>(st, b, adj) && !(g_fx_corrections && st.var[2 + g_tc_mode][adj ? 1 : 0][rhs_bucket(b)] == 0);
+}
+
 template <typename V>
 void launch_stage(const Stage& st, bool adj, const V* x, long long xrs, long long xcs, V* y,
                   long long yrs, long long ycs, int b, cudaStream_t s) {
-  if (st.nblk == 0) return;
-  if (use_tc<V>(st, b, adj)) {
+  if (st.nblk == 0 || launch_correction<V>(st, adj, x, xrs, xcs, y, yrs, ycs, b, s)) return;
+  if (tc_serves<V>(st, b, adj)) {
     const int tv = st.var[2 + g_tc_mode][adj ? 1 : 0][rhs_bucket(b)];
     if (tv != kFp32CoresVariant) {
       if (!launch_tc(st, adj, (const float2*)x, xrs, xcs, (float2*)y, yrs, ycs, b, s, tv))
@@ -1156,7 +1172,7 @@ template <>
 bool inplace_split<float2>(const Stage& st, bool adj, float2* W, float2* P, long long pcap, int b, int rs, cudaStream_t s) {
   if (!P) return false;
   const int bk = rhs_bucket(b), dir = adj ? 1 : 0;
-  const bool tc = use_tc<float2>(st, b, adj);
+  const bool tc = tc_serves<float2>(st, b, adj);
   const bool dflt = split_by_default(st, adj, b);
   if (!tc || st.var[2 + g_tc_mode][dir][bk] == kFp32CoresVariant) {
     const int v = st.var[1][dir][bk];
@@ -1193,11 +1209,11 @@ template <typename V>
 void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, int rs, cudaStream_t s, V* P = nullptr,
                    long long pcap = 0) {
   if (st.nblk == 0) return;
-  if (inplace_split<V>(st, adj, W, P, pcap, b, rs, s)) {
+  // the fixed-point kernel reads W in a launch of its own (the gather), so it may write W
+  if (launch_correction<V>(st, adj, W, rs, 1, W, rs, 1, b, s) || inplace_split<V>(st, adj, W, P, pcap, b, rs, s)) {
     mark(s);
     return;
   }
-  // the fixed-point kernel reads W in a launch of its own (the gather), so it may write W
   const int var = st.var[type_index<V>()][adj ? 1 : 0][rhs_bucket(b)];
   if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, W, rs, 1, W, rs, 1, b, s, var == kFxVariant)) {
     mark(s);
@@ -1384,7 +1400,7 @@ int fio_tc_timeout_reset() {
 
 int fio_apply_correction(fio_op op, int which, const void* x, void* y, int64_t ld, int b, cudaStream_t s) {
   g_fx_corrections = true;
-  const int rc = fio_apply_internal(op, which, x, y, ld, b, FIO_P32, s);
+  const int rc = fio_apply_internal(op, which, x, y, ld, b, FIO_PTF32X3, s);
   g_fx_corrections = false;
   return rc;
 }
@@ -1632,6 +1648,7 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
         if (rc == FIO_OK && (tc || best == kFxVariant) && fio_tc_timeout_reset() != 0) rc = FIO_ETIMEOUT;
       }
       st.var[ti][dir][bucket] = (int8_t)best;
+      if (tc && g_tc_mode == kTcX3) st.x3_pinned[bucket] = false;
       if (choices && n < cap) choices[n] = best;
       ++n;
     }
@@ -1663,7 +1680,10 @@ extern "C" int fio_set_variant(fio_op op, int b, int precision, int variant) {
         (is_3m_variant(variant) && ti == 1))
       return FIO_EINVAL;
   }
-  for (auto& st : op->st) st.var[ti][0][bucket] = st.var[ti][1][bucket] = (int8_t)variant;
+  for (auto& st : op->st) {
+    st.var[ti][0][bucket] = st.var[ti][1][bucket] = (int8_t)variant;
+    if (tc && mode == kTcX3) st.x3_pinned[bucket] = variant != 0;
+  }
   return FIO_OK;
 }
 

@@ -52,6 +52,7 @@ struct Stage {
   // kernel variant chosen by fio_autotune per [arithmetic: c128, c64, double-float, TF32, BF16,
   // split TF32][direction: forward, adjoint][right-hand-side bucket]; 0 = the built-in choice
   // (see fio_capi.cu)
+  bool x3_pinned[5] = {};  // per bucket: the split-TF32 variant was set by fio_set_variant, not by the autotuner
   int8_t var[6][2][5] = {};
   // TMA tensor maps of the tensor-core A operands per [direction: forward (M32 / Mbf), adjoint
   // (M32t / Mbft)][element: FP32, BF16]; tma_ok marks the maps that encoded (16-byte aligned
@@ -166,8 +167,9 @@ int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void
 // which: 0 K-dot, 1 K-dot*, 2 G-dot, 3 G-dot K-dot*; x, y column-major with leading dimension ld
 int fio_apply_internal(fio_op op, int which, const void* x, void* y, int64_t ld, int b, int prec,
                        cudaStream_t s);
-// the same in FP32 for a correction asked for in split TF32: large stages in 30-bit fixed point (closer than
-// split TF32, faster than the FP32 CUDA cores)
+// the same for a correction asked for in split TF32: stages with work enough in 30-bit fixed point (closer
+// than split TF32, and faster) unless a variant is pinned for split TF32, the others in what is tuned or pinned
+// for split TF32, or else on the FP32 CUDA cores
 int fio_apply_correction(fio_op op, int which, const void* x, void* y, int64_t ld, int b, cudaStream_t s);
 void fio_solver_free(fio_op op);
 // 1 when a tensor-core kernel's bounded wait gave up since the last call (and clear the flag),

@@ -214,6 +214,7 @@ struct Ctx {
   double2* host;        // pinned scalars (dots)
   int outer = FIO_P64;  // precision of the true residuals (FIO_P64 or FIO_PDF)
   bool f_zero = false;  // f is known to be zero (the next residual is u itself)
+  bool direct = false;  // FIO_DIRECT
 };
 
 int dots(Ctx& c, const double2* a, long long lda, const double2* bb, long long ldb, double2* out_dev,
@@ -252,10 +253,8 @@ inline double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 // G-dot x (which = 2); x, y FP64 with ld = N
 int precond(Ctx& c, Work& w, int which, const double2* x, double2* y, int prec) {
   if (prec == FIO_P64) return fio_apply_internal(c.op, which, x, y, c.N, c.b, FIO_P64, c.s);
-  // split-TF32 corrections run in FP32: closer to the factors' product (7e-7 against 2.6e-5 on the 2D
-  // n = 256 shapes), and since its large stages are on the tensor cores too, faster (2D n = 128, b = 32:
-  // 0.33 ms an apply against 0.45; n = 256 2.4 against 3.2)
-  const bool split = prec == FIO_PTF32X3;
+  // FIO_DIRECT gives the answer itself, in the arithmetic that was asked for
+  const bool split = prec == FIO_PTF32X3 && !c.direct;
   const long long n = c.N * c.b;
   pdl_launch(true, k_to32, nblocks(n), 256, 0, c.s, x, w.v32[0], n);
   int rc = split ? fio_apply_correction(c.op, which, w.v32[0], w.v32[1], c.N, c.b, c.s)
@@ -325,6 +324,7 @@ extern "C" int fio_solve(fio_op op, const void* uv, void* fv, int64_t ld, int b,
   if (rc) return rc;
   Ctx c{op, rop, op->N, b, s, w.host};
   c.outer = opts->outer;
+  c.direct = opts->method == FIO_DIRECT;
   const double2* u = (const double2*)uv;
   double2* f = (double2*)fv;
   const long long N = op->N;
