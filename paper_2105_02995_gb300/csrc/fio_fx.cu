@@ -82,7 +82,10 @@ bool launch(FxArgs a, uint8_t* X, int* ej, cudaStream_t s) {
   // 1D N = 16384 b = 5, 15 K steps: 414 us without, 360 with)
   const bool early = (long long)a.steps * a.nrt <= 300LL * sm_count();
   const int groups = (a.maxcols + 4 * (256 / BT) - 1) / (4 * (256 / BT));
-  auto gather = groups <= 1 ? k_fx_gather<R, ADJ, BT, 1> : groups <= 2 ? k_fx_gather<R, ADJ, BT, 2> : k_fx_gather<R, ADJ, BT, 4>;
+  auto gather = groups <= 1   ? k_fx_gather<R, ADJ, BT, 1>
+                : groups <= 2 ? k_fx_gather<R, ADJ, BT, 2>
+                : groups <= 4 ? k_fx_gather<R, ADJ, BT, 4>
+                              : k_fx_gather<R, ADJ, BT, 0>;
   pdl_launch(early, gather, dim3((unsigned)a.nblk, (unsigned)a.nrt), 256, 0, s, a, X, ej);
   pdl_launch(true, k_stage_fx<R, ADJ, BT>, (unsigned)std::min<long long>(total, sm_count()), fx::kThreads, need, s, a);
   return true;

@@ -333,8 +333,8 @@ template <int I> using Int = std::integral_constant<int, I>;
 // The gathered vector of every block as digits (layout above), and its columns' scale exponents.
 // A CTA per (block, right-hand-side tile), a thread for every CS-th group of four columns of one
 // right-hand side.  Bound by the latency of its two dependent loads, list and vector: the entries of
-// up to HOLD groups stay in registers between the maximum and the cut (blocks of at most 4 CS HOLD columns;
-// no more than a stage needs, for the registers), longer blocks load them twice.
+// up to HOLD groups stay in registers between the maximum and the cut (stages of at most 4 CS HOLD columns a
+// block; no more than a stage needs, for the registers), those of longer blocks are loaded twice (HOLD 0).
 template <typename R, bool ADJ, int BT, int HOLD>
 __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, int* ej) {
   using namespace fx;
@@ -376,11 +376,11 @@ __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, i
     for (int i = 0; i < 4; ++i) m = max(m, scale_key(f.v[i], f.ce[i]));
     return m;
   };
-  const bool hold = HOLD < 4 || nq <= HOLD * CS;  // HOLD 1 and 2 are launched for stages that fit
-  Four held[HOLD];
-  int4 lp[HOLD], lq[HOLD];
+  constexpr bool hold = HOLD > 0;
+  Four held[HOLD + 1];
+  int4 lp[HOLD + 1], lq[HOLD + 1];
   const int4 none = make_int4(-1, 0, -1, 0);
-  if (hold) {
+  if constexpr (hold) {
 #pragma unroll
     for (int k = 0; k < HOLD; ++k) {
       const int q = c0 + k * CS;
@@ -391,13 +391,13 @@ __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, i
   __syncthreads();
   pdl_wait();
   int m = 0;
-  if (hold) {
+  if constexpr (hold) {
 #pragma unroll
     for (int k = 0; k < HOLD; ++k) get(held[k], lp[k], lq[k]);
 #pragma unroll
     for (int k = 0; k < HOLD; ++k) m = key(held[k], m);
   } else {
-#pragma unroll 4
+#pragma unroll 1
     for (int q = c0; q < nq; q += CS) {
       Four f;
       get(f, list[2 * q], list[2 * q + 1]);
@@ -435,12 +435,12 @@ __global__ void __launch_bounds__(256) k_fx_gather(const FxArgs a, uint8_t* X, i
       o[6 * wt] = digit_pair<3>(re, im);
     }
   };
-  if (hold) {
+  if constexpr (hold) {
 #pragma unroll
     for (int k = 0; k < HOLD; ++k)
       if (c0 + k * CS < nq) put(c0 + k * CS, held[k]);
   } else {
-#pragma unroll 2
+#pragma unroll 1
     for (int q = c0; q < nq; q += CS) {
       Four f;
       get(f, list[2 * q], list[2 * q + 1]);
