@@ -31,7 +31,8 @@
  * to the FP32 CUDA-core kernels.  The large stages of FIO_P64 (and of FIO_P32 under variant 50) run on the tensor cores in
  * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below their row's and column's largest,
  * digit products summed exactly, each output rounded once (columns with infinities, NaN or extreme exponents are summed plainly).  The
- * digit copies that this takes are made at upload where they fit half of the free device memory.
+ * digit copies that this takes (FP32's with FIO_MASK_TC only) are made at upload where they fit half of the
+ * free device memory, FP64's first.
  * fio_solve's corrections with inner = FIO_PTF32X3 take them too (see there).
  * FIO_PDF takes complex128 vectors and applies a double-float copy
  * of the factors (each FP64 entry as an unevaluated sum of two floats, 48-bit significand) with

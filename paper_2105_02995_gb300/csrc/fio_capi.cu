@@ -1326,11 +1326,20 @@ void apply_core(fio_op op, Which w, const V* x, V* y, int64_t ld, int b, V* A, V
   }
 }
 
+// whether a call may launch the fixed-point kernel, and takes its scratch
+bool fx_may_run(fio_op op, int b, size_t elem) {
+  if (elem != sizeof(float2) || g_fx_corrections) return true;
+  for (const auto& st : op->st)
+    for (int dir = 0; dir < 2; ++dir)
+      if (st.var[1][dir][rhs_bucket(b)] == kFxVariant) return true;
+  return false;
+}
+
 template <typename V>
 int apply_t(fio_op op, Which w, const void* xv, void* yv, int64_t ld, int b, cudaStream_t s) {
-  void *bufs[5], *fxb;
-  size_t fxn;
-  int rc = fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn);
+  void *bufs[5], *fxb = nullptr;
+  size_t fxn = 0;
+  int rc = fx_may_run(op, b, sizeof(V)) ? fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn) : fio_scratch(op, b, sizeof(V), s, bufs);
   if (rc) return rc;
   FxScratch fxs(fxb, fxn);
   apply_core<V>(op, w, (const V*)xv, (V*)yv, ld, b, (V*)bufs[0], (V*)bufs[1], (V*)bufs[2], s);
@@ -1449,7 +1458,7 @@ extern "C" int fio_apply_inv_host(fio_op op, const void* u_host, void* f_host, i
   cudaStream_t s = (cudaStream_t)stream;
   const size_t es = dtype == FIO_C128 ? 16 : 8;
   void *bufs[5], *fxb;  // asked for with its scratch, so that the apply below does not grow it again
-  int rc = fio_scratch(op, b, es, s, bufs, &fxb);
+  int rc = fio_scratch(op, b, es, s, bufs, fx_may_run(op, b, es) ? &fxb : nullptr);
   if (rc) return rc;
   void *U = bufs[3], *F = bufs[4];
   const size_t w = (size_t)op->N * es;
@@ -1569,9 +1578,9 @@ constexpr int kTcCand[9] = {0,  20, 21, 22, kTmaVariant, kTmaSplitVariant, kTmaB
 // per (stage, direction) in stage order, forward before adjoint
 template <typename V>
 int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch) {
-  void *bufs[5], *fxb;
-  size_t fxn;
-  int rc = fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn);
+  void *bufs[5], *fxb = nullptr;
+  size_t fxn = 0;
+  int rc = fio_scratch(op, b, sizeof(V), s, bufs, sizeof(V) == sizeof(float2) ? nullptr : &fxb, &fxn);
   if (rc) return rc;
   FxScratch fxs(fxb, fxn);
   const int rs = row_stride<V>(b);

@@ -102,7 +102,8 @@ bool launch_b(const FxArgs& a, uint8_t* X, int* ej, cudaStream_t s) {
 }  // namespace
 
 int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>& mdims, cudaStream_t s) {
-  const bool want[2] = {(op->mask & FIO_MASK_P64) != 0, (op->mask & FIO_MASK_P32) != 0 && op->arena32};
+  // (the FP32 copies serve the corrections asked for in split TF32, and variant 50 when it is pinned)
+  bool want[2] = {(op->mask & FIO_MASK_P64) != 0, op->arena32 && op->arena_tc};
   if (!want[0] && !want[1]) return FIO_OK;
   struct Plan {
     int stage;
@@ -112,7 +113,7 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
   std::vector<Plan> plans;
   std::vector<FxUnit> units;
   std::vector<int2> xofs;
-  size_t nexp = 0, nlist = 0, dbytes = 0;
+  size_t nexp = 0, nlist = 0, dbytes[2] = {0, 0};
   for (size_t si = 0; si < op->st.size(); ++si) {
     Stage& st = op->st[si];
     int2 n = make_int2(0, 0);
@@ -177,10 +178,11 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
     }
     for (int t = 0; t < 2; ++t)
       for (int dir = 0; p.want[t] && dir < 2; ++dir) {
-        p.digits[t][dir] = dbytes;
-        dbytes += al256(bytes[t][dir]);
+        p.digits[t][dir] = dbytes[t];
+        dbytes[t] += al256(bytes[t][dir]);
       }
-    for (int t = 0; t < 2; ++t) op->fx_max_cols[t] = std::max(op->fx_max_cols[t], cols[t]);
+    for (int t = 0; t < 2; ++t)
+      if (p.want[t]) op->fx_max_cols[t] = std::max(op->fx_max_cols[t], cols[t]);
     op->fx_max_blk = std::max(op->fx_max_blk, (long long)st.nblk);
     plans.push_back(p);
   }
@@ -189,17 +191,27 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
                ol = ox + al256(xofs.size() * sizeof(int2)), ob = ol + al256(nlist * sizeof(int2)),
                od = ob + al256(plans.size() * sizeof(int));
   // The copies take at most half of the free memory, so that scratch, solver vectors and other operators
-  // find the room they had without them; where they do not fit, the CUDA-core kernels serve.
+  // find the room they had without them: both types', or FP64's alone, or none (the CUDA-core kernels serve).
   size_t room = 0, all = 0;
-  if (cudaMemGetInfo(&room, &all) != cudaSuccess || od + dbytes > room / 2 ||
-      cudaMalloc(&op->fx, od + dbytes) != cudaSuccess) {
-    cudaGetLastError();
-    op->fx = nullptr;
-    op->fx_max_cols[0] = op->fx_max_cols[1] = 0;
-    return FIO_OK;
+  if (cudaMemGetInfo(&room, &all) != cudaSuccess) room = 0;
+  cudaGetLastError();
+  for (const bool both : {true, false}) {
+    const size_t bytes = od + dbytes[0] + (both ? dbytes[1] : 0);
+    if (op->fx || bytes == od || bytes > room / 2) continue;
+    if (cudaMalloc(&op->fx, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      op->fx = nullptr;
+      continue;
+    }
+    op->fx_bytes = bytes;
+    want[1] = want[1] && both;
   }
-  op->fx_bytes = od + dbytes;
-  uint8_t* p0 = (uint8_t*)op->fx;
+  if (!op->fx) want[0] = want[1] = false;
+  for (int t = 0; t < 2; ++t)
+    if (!want[t]) op->fx_max_cols[t] = 0;
+  if (!op->fx) return FIO_OK;
+  for (Plan& p : plans) p.want[1] = p.want[1] && want[1];
+  uint8_t *p0 = (uint8_t*)op->fx, *pd[2] = {p0 + od, p0 + od + dbytes[0]};
   int* bad = (int*)(p0 + ob);
   if (cudaMemcpyAsync(p0, units.data(), units.size() * sizeof(FxUnit), cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemcpyAsync(p0 + ox, xofs.data(), xofs.size() * sizeof(int2), cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -222,15 +234,15 @@ int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>
       st.fx_list[dir] = list;
       st.fx_units[dir] = (const FxUnit*)p0 + p.units[dir];
       st.fx_xofs[dir] = (const int2*)(p0 + ox) + p.xofs[dir];
-      for (int t = 0; t < 2; ++t) st.fxA[t][dir] = p.want[t] ? p0 + od + p.digits[t][dir] : nullptr;
+      for (int t = 0; t < 2; ++t) st.fxA[t][dir] = p.want[t] ? pd[t] + p.digits[t][dir] : nullptr;
     }
     if (p.want[0]) {
-      pack<double, false>(st, st.fx_units[0], p0 + od + p.digits[0][0], s);
-      pack<double, true>(st, st.fx_units[1], p0 + od + p.digits[0][1], s);
+      pack<double, false>(st, st.fx_units[0], pd[0] + p.digits[0][0], s);
+      pack<double, true>(st, st.fx_units[1], pd[0] + p.digits[0][1], s);
     }
     if (p.want[1]) {
-      pack<float, false>(st, st.fx_units[0], p0 + od + p.digits[1][0], s);
-      pack<float, true>(st, st.fx_units[1], p0 + od + p.digits[1][1], s);
+      pack<float, false>(st, st.fx_units[0], pd[1] + p.digits[1][0], s);
+      pack<float, true>(st, st.fx_units[1], pd[1] + p.digits[1][1], s);
     }
   }
   std::vector<int> hbad(plans.size(), 1);
