@@ -407,6 +407,7 @@ extern "C" int fio_release(fio_op op) {
   if (op->fft_tw) cudaFree(op->fft_tw);
   if (op->arena_tc) cudaFree(op->arena_tc);
   if (op->scratch) cudaFree(op->scratch);
+  if (op->fx_scratch) cudaFree(op->fx_scratch);
   if (op->flag_host) cudaFreeHost(op->flag_host);
   fio_solver_free(op);
   cudaGetLastError();
@@ -421,7 +422,8 @@ extern "C" int fio_query(fio_op op, int* d, int64_t* n, int64_t* N, size_t* devi
   if (N) *N = op->N;
   if (device_bytes)
     *device_bytes = op->arena_bytes + op->arena32_bytes + op->arena_tc_bytes + op->arena_df_bytes + op->meta_bytes +
-                    op->units_bytes + op->fx_bytes + op->fft_bytes + op->scratch_bytes + op->solver_bytes;
+                    op->units_bytes + op->fx_bytes + op->fft_bytes + op->scratch_bytes +
+                    op->fx_scratch_bytes + op->solver_bytes;
   return FIO_OK;
 }
 
@@ -445,33 +447,38 @@ extern "C" const char* fio_strerror(int status) {
 int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void** fxbuf, size_t* fxbytes) {
   const size_t per = (size_t)op->max_len * (size_t)(elem == 8 ? (b + 1) & ~1 : b) * elem;  // row_stride
   const size_t per_al = (per + 255) & ~(size_t)255;
-  size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
-  size_t need = 5 * per_al + fxneed;
-  if (need > op->scratch_bytes) {
-    if (op->scratch) {
+  // FIO_OK, FIO_ENOMEM (the buffer is gone) or FIO_ECUDA
+  auto grow = [&](void** buf, size_t* bytes, size_t need) {
+    if (need <= *bytes) return FIO_OK;
+    if (*buf) {
       if (cudaStreamSynchronize(s) != cudaSuccess) return FIO_ECUDA;
-      cudaFree(op->scratch);
-      op->scratch = nullptr;
-      op->scratch_bytes = 0;
+      cudaFree(*buf);
+      *buf = nullptr;
+      *bytes = 0;
     }
-    bool got = cudaMalloc(&op->scratch, need) == cudaSuccess;
-    if (!got && fxneed) {  // without the fixed-point kernel's part, from now on: the CUDA-core kernels serve
+    if (cudaMalloc(buf, need) != cudaSuccess) {
       cudaGetLastError();
-      fx_give_up(op, elem);
-      fxneed = 0;
-      need = 5 * per_al;
-      got = cudaMalloc(&op->scratch, need) == cudaSuccess;
-    }
-    if (!got) {
-      cudaGetLastError();
-      op->scratch = nullptr;
+      *buf = nullptr;
       return FIO_ENOMEM;
     }
-    op->scratch_bytes = need;
+    *bytes = need;
+    return FIO_OK;
+  };
+  int rc = grow(&op->scratch, &op->scratch_bytes, 5 * per_al);
+  if (rc == FIO_ENOMEM && op->fx_scratch) {  // what the fixed-point kernel holds may be what is missing
+    cudaFree(op->fx_scratch);
+    op->fx_scratch = nullptr;
+    op->fx_scratch_bytes = 0;
+    rc = grow(&op->scratch, &op->scratch_bytes, 5 * per_al);
   }
+  if (rc) return rc;
   for (int k = 0; k < 5; ++k) bufs[k] = (uint8_t*)op->scratch + k * per_al;
-  if (fxbuf) *fxbuf = fxneed ? (uint8_t*)op->scratch + 5 * per_al : nullptr;
-  if (fxbytes) *fxbytes = fxneed;
+  // no room for the fixed-point kernel's: this call runs on the CUDA cores
+  const size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
+  rc = fxneed ? grow(&op->fx_scratch, &op->fx_scratch_bytes, fxneed) : FIO_ENOMEM;
+  if (rc == FIO_ECUDA) return rc;
+  if (fxbuf) *fxbuf = rc == FIO_OK ? op->fx_scratch : nullptr;
+  if (fxbytes) *fxbytes = rc == FIO_OK ? fxneed : 0;
   return FIO_OK;
 }
 
@@ -1786,7 +1793,10 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
             cudaMalloc(&acc, 2 * sizeof(double)) == cudaSuccess;
   const size_t fxn = std::max(fx_scratch_bytes(op, b, sizeof(double2)), fx_scratch_bytes(op, b, sizeof(float2)));
   void* fxb = nullptr;
-  if (ok && fxn) ok = cudaMalloc(&fxb, fxn) == cudaSuccess;
+  if (ok && fxn && cudaMalloc(&fxb, fxn) != cudaSuccess) {  // no room: the CUDA cores serve
+    cudaGetLastError();
+    fxb = nullptr;
+  }
   FxScratch fxs(fxb, fxn);
   int rc = ok ? FIO_OK : FIO_ENOMEM;
   int k = 0;

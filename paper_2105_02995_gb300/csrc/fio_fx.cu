@@ -289,8 +289,6 @@ bool fx_takes(const Stage& st, bool adj, bool wide, int b) {
   return b > 8 && units >= 2LL * sms && fx < 8e-6 * (double)st.nnz * bp / (b <= 16 ? 31.0 : 42.0);
 }
 
-void fx_give_up(fio_op op, size_t elem) { op->fx_max_cols[elem == sizeof(double2) ? 0 : 1] = 0; }
-
 bool fx_all_wide(fio_op op) {
   if (op->fx_max_cols[0] == 0) return false;
   for (const Stage& st : op->st)

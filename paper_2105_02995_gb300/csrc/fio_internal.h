@@ -105,6 +105,8 @@ struct fio_op_s {
   size_t fx_bytes = 0;
   long long fx_max_cols[2] = {0, 0};  // most columns of a gathered vector (FP64, FP32 chunking)
   long long fx_max_blk = 0;           // most blocks of a stage it takes
+  void* fx_scratch = nullptr;         // its scratch, apart from the pool: a call runs without it where it has no room
+  size_t fx_scratch_bytes = 0;
   void* fft_tw = nullptr;         // DFT twiddles: exp(2 pi i k / 2048), 2048 double2 then 2048 float2
   size_t fft_bytes = 0;
   void* solver = nullptr;         // solver work arrays (fio_solve.cu)
@@ -153,7 +155,6 @@ inline bool is_tc_precision(int p) { return p == FIO_PTF32 || p == FIO_PBF16 || 
 // launch; the launch (false: not taken, nothing launched; *timeout is set by a bounded wait that gives up)
 int fx_build(fio_op op, const std::vector<int2>& meta, const std::vector<size_t>& mdims, cudaStream_t s);
 size_t fx_scratch_bytes(fio_op op, int b, size_t elem);
-void fx_give_up(fio_op op, size_t elem);  // no room for that scratch: the type's launches keep the other kernels
 bool fx_takes(const fio::Stage& st, bool adj, bool wide, int b);
 int fft_build(fio_op op, cudaStream_t s);  // the DFT's twiddle table (fio_fft.cu)
 bool fx_all_wide(fio_op op);  // every stage of the operator has an FP64 digit copy
@@ -161,7 +162,7 @@ bool fx_launch(const fio::Stage& st, bool adj, bool wide, const void* x, long lo
                long long yrs, long long ycs, int b, void* scratch, size_t scratch_bytes, int* timeout, cudaStream_t s);
 
 // scratch work arrays (5 of max_len x b elements of `elem` bytes); grows with a stream sync;
-// fxbuf (may be null) receives the fixed-point kernel's scratch behind them, fxbytes its size
+// fxbuf (may be null) receives the fixed-point kernel's scratch, or null where there is no room, fxbytes its size
 int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void** fxbuf = nullptr,
                 size_t* fxbytes = nullptr);
 // which: 0 K-dot, 1 K-dot*, 2 G-dot, 3 G-dot K-dot*; x, y column-major with leading dimension ld

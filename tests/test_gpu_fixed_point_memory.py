@@ -86,3 +86,24 @@ def test_fp64_copies_come_first(packed):
     assert held(op) < arenas + DIGITS64 + DIGITS32 // 2
     assert torch.equal(op.apply_K(x), want)
     op.release()
+
+
+def test_scratch_that_does_not_fit_is_asked_for_again(packed):
+    """One call without room for the fixed-point scratch runs on the CUDA cores; the calls after it do not."""
+    op, wide = binding.Operator(packed), 96
+    x8, x = vectors(8, torch.complex128), vectors(wide, torch.complex128)
+    want8, out = op.apply_K(x8), binding.colmajor(torch.empty_like(x))
+    op.set_variant(wide, binding.FIO_P64, 1)
+    cores = op.apply_K(x)
+    op.set_variant(wide, binding.FIO_P64, 0)
+    op.release()
+    op = binding.Operator(packed)
+    pool = 5 * 16 * N * wide  # and 1/5 of it for the fixed-point kernel
+    with Hog(pool + pool // 10):
+        op.apply_K(x, out)
+        torch.cuda.synchronize()
+        assert held(op) >= pool
+    assert torch.equal(out, cores)
+    assert torch.equal(op.apply_K(x8), want8)
+    assert not torch.equal(op.apply_K(x, out), cores)
+    op.release()
