@@ -40,8 +40,8 @@
  * (~1e-14 relative per stage) at the FP32 pipes' rate, for the outer residual of iterative
  * refinement (GB300's FP64 rate is a small fraction of its FP32 rate); it adds two conversion
  * launches per apply and is not accepted by fio_apply_inv_noalloc.  Where every stage of the operator
- * runs in fixed point (operators above 4096 unknowns with both copies), FIO_PDF runs as FIO_P64: more
- * accurate than double-float, and faster.  The vector dtype
+ * runs in fixed point (operators above 4096 unknowns with both copies), FIO_PDF runs in FP64: more
+ * accurate than double-float, and faster; its kernel choices are its own, not FIO_P64's.  The vector dtype
  * must match the precision (C128 with P64 and PDF, C64 with the others); other pairs return FIO_EINVAL.
  *
  * STREAMS AND SCRATCH.  Calls are asynchronous on `stream` (a cudaStream_t; NULL = the legacy
@@ -251,7 +251,7 @@ int fio_set_variant(fio_op op, int b, int precision, int variant);
  * HIF stage and the root) stores ||y_p - y_64|| / ||y_64|| of the intermediate vectors in
  * errs_host[k] (k < cap), in application order; *nerr receives the number of stages.  The FP64
  * path is the one held to 1e-12 of the oracle, so these are errors against the oracle's
- * arithmetic.  Allocates its own work vectors and synchronises `stream`. */
+ * arithmetic (beside FIO_PDF in FP64 fixed point it runs on the CUDA cores).  Allocates its own work vectors and synchronises `stream`. */
 int fio_stage_errors(fio_op op, int which, const void* x, int64_t ld, int b, int precision, void* stream,
                      double* errs_host, int cap, int* nerr);
 

@@ -1015,6 +1015,16 @@ template <> constexpr int type_index<double2>() { return 0; }
 template <> constexpr int type_index<float2>() { return 1; }
 template <> constexpr int type_index<dfc>() { return 2; }
 
+// FIO_PDF running in FP64 (df_as_fp64): its choices are kept apart from FIO_P64's
+thread_local bool g_for_df = false;
+struct ForDf {
+  bool prev;
+  explicit ForDf(bool on) : prev(g_for_df) { g_for_df = on; }
+  ~ForDf() { g_for_df = prev; }
+};
+template <typename V>
+int var_table() { return std::is_same<V, double2>::value && g_for_df ? 6 : type_index<V>(); }
+
 template <typename V>
 StageArgs<V> stage_args(const Stage& st, bool adj, const V* x, long long xrs, long long xcs, V* y,
                         long long yrs, long long ycs, int b) {
@@ -1125,7 +1135,7 @@ void launch_stage(const Stage& st, bool adj, const V* x, long long xrs, long lon
     }
   }
   const StageArgs<V> a = stage_args<V>(st, adj, x, xrs, xcs, y, yrs, ycs, b);
-  int var = st.var[type_index<V>()][adj ? 1 : 0][rhs_bucket(b)];
+  int var = st.var[var_table<V>()][adj ? 1 : 0][rhs_bucket(b)];
   if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, x, xrs, xcs, y, yrs, ycs, b, s, var == kFxVariant)) return;
   if (st.kind == 1) var = four_product_of(var);  // in-place stages keep four products
   if (adj) launch_stage_dir<V, true>(a, s, var);
@@ -1221,7 +1231,7 @@ void inplace_stage(const Stage& st, bool adj, V* W, V* S, int b, int rs, cudaStr
     mark(s);
     return;
   }
-  const int var = st.var[type_index<V>()][adj ? 1 : 0][rhs_bucket(b)];
+  const int var = st.var[var_table<V>()][adj ? 1 : 0][rhs_bucket(b)];
   if ((var == 0 || var == kFxVariant) && launch_fx<V>(st, adj, W, rs, 1, W, rs, 1, b, s, var == kFxVariant)) {
     mark(s);
     return;
@@ -1342,12 +1352,15 @@ bool fx_may_run(fio_op op, int b, size_t elem) {
   return false;
 }
 
+constexpr int kNoRoom = 1;  // FIO_PDF in FP64: no room for the fixed-point scratch (never returned to a caller)
+
 template <typename V>
 int apply_t(fio_op op, Which w, const void* xv, void* yv, int64_t ld, int b, cudaStream_t s) {
   void *bufs[5], *fxb = nullptr;
   size_t fxn = 0;
   int rc = fx_may_run(op, b, sizeof(V)) ? fio_scratch(op, b, sizeof(V), s, bufs, &fxb, &fxn) : fio_scratch(op, b, sizeof(V), s, bufs);
   if (rc) return rc;
+  if (g_for_df && !fxb) return kNoRoom;
   FxScratch fxs(fxb, fxn);
   apply_core<V>(op, w, (const V*)xv, (V*)yv, ld, b, (V*)bufs[0], (V*)bufs[1], (V*)bufs[2], s);
   return finish(s);
@@ -1370,8 +1383,9 @@ int apply_df(fio_op op, Which w, const void* xv, void* yv, int64_t ld, int b, cu
 
 // Whether FIO_PDF runs as FIO_P64: when every stage has the fixed-point kernel's FP64 copy, that
 // kernel is both faster than double-float arithmetic on the FP32 pipes (2D n = 256, K-dot at b = 16:
-// 3.4 ms against 15) and more accurate (exact sums of 62-bit operands against 48-bit ones).  A
-// double-float variant pinned by fio_set_variant keeps the double-float kernels.
+// 3.1 ms against 15) and more accurate (exact sums of 62-bit operands against 48-bit ones).  A
+// double-float variant pinned by fio_set_variant keeps the double-float kernels, as does a call that
+// has no room for the fixed-point scratch.
 bool df_as_fp64(fio_op op, int b) {
   if (!fx_all_wide(op)) return false;
   const int k = rhs_bucket(b);
@@ -1381,7 +1395,12 @@ bool df_as_fp64(fio_op op, int b) {
 }
 
 int apply_prec(fio_op op, Which w, const void* x, void* y, int64_t ld, int b, int prec, cudaStream_t s) {
-  if (prec == FIO_P64 || (prec == FIO_PDF && df_as_fp64(op, b))) return apply_t<double2>(op, w, x, y, ld, b, s);
+  if (prec == FIO_P64) return apply_t<double2>(op, w, x, y, ld, b, s);
+  if (prec == FIO_PDF && df_as_fp64(op, b)) {
+    ForDf in_fp64(true);
+    const int rc = apply_t<double2>(op, w, x, y, ld, b, s);
+    if (rc != kNoRoom) return rc;
+  }
   if (prec == FIO_PDF) return apply_df(op, w, x, y, ld, b, s);
   TcMode m(tc_mode_of(prec));
   return apply_t<float2>(op, w, x, y, ld, b, s);
@@ -1589,6 +1608,7 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
   size_t fxn = 0;
   int rc = fio_scratch(op, b, sizeof(V), s, bufs, sizeof(V) == sizeof(float2) ? nullptr : &fxb, &fxn);
   if (rc) return rc;
+  if (g_for_df && !fxb) return kNoRoom;
   FxScratch fxs(fxb, fxn);
   const int rs = row_stride<V>(b);
   const size_t bytes = (size_t)op->max_len * rs * sizeof(V);
@@ -1611,9 +1631,11 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
     for (int dir = 0; dir < (root ? 1 : 2) && rc == FIO_OK; ++dir) {
       const bool adj = dir == 1;
       const bool tc = use_tc<V>(st, b, adj);
-      const int ti = tc ? 2 + g_tc_mode : type_index<V>();
+      const int ti = tc ? 2 + g_tc_mode : var_table<V>();
       int best = 0;
-      if (st.nblk > 0) {
+      if (g_for_df && fx_takes(st, adj, true, b)) {
+        best = kFxVariant;  // what FIO_PDF runs in FP64 for: several times as fast as the CUDA-core tiles
+      } else if (st.nblk > 0) {
         const StageArgs<V> a = stage_args<V>(st, adj, X, rs, 1, Y, rs, 1, b);
         float tbest = -1.f;
         const int ncand = tc ? 9 : kNCand + 1;
@@ -1698,6 +1720,7 @@ extern "C" int fio_set_variant(fio_op op, int b, int precision, int variant) {
   }
   for (auto& st : op->st) {
     st.var[ti][0][bucket] = st.var[ti][1][bucket] = (int8_t)variant;
+    if (ti == 2) st.var[6][0][bucket] = st.var[6][1][bucket] = 0;
     if (tc && mode == kTcX3) st.x3_pinned[bucket] = variant != 0;
   }
   return FIO_OK;
@@ -1722,10 +1745,15 @@ extern "C" int fio_autotune(fio_op op, int b, int precision, void* stream, int* 
   }
   g_tune_flush = flush;
   int rc;
-  if (precision == FIO_P64 || (precision == FIO_PDF && df_as_fp64(op, b))) {
+  if (precision == FIO_P64) {
     rc = tune_type<double2>(op, b, s, choices, cap, nchoices);
   } else if (precision == FIO_PDF) {
-    rc = tune_type<dfc>(op, b, s, choices, cap, nchoices);
+    rc = kNoRoom;
+    if (df_as_fp64(op, b)) {
+      ForDf in_fp64(true);
+      rc = tune_type<double2>(op, b, s, choices, cap, nchoices);
+    }
+    if (rc == kNoRoom) rc = tune_type<dfc>(op, b, s, choices, cap, nchoices);
   } else {
     TcMode m(tc_mode_of(precision));
     rc = tune_type<float2>(op, b, s, choices, cap, nchoices);
@@ -1813,6 +1841,13 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
     if (k < cap) errs[k] = h[1] > 0.0 ? sqrt(h[0] / h[1]) : sqrt(h[0]);
     ++k;
   };
+  // the FP64 chain beside FIO_PDF in FP64 runs on the CUDA cores: not the kernel that is measured
+  auto reference = [&](auto&& launch) {
+    const bool other = std::is_same<V, double2>::value;
+    ForDf plain(g_for_df && !other);
+    FxScratch cores(other ? nullptr : g_fx_scratch, other ? 0 : g_fx_bytes);
+    launch();
+  };
   if (rc == FIO_OK) {
     const long long N = op->N;
     to_row<double2>((const double2*)x, ld, W64, N, b, b, s);  // both chains start from the same values
@@ -1825,7 +1860,7 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
         const Stage& st = op->st[adj ? op->n_bf - 1 - kk : kk];
         double2* d64 = (kk & 1) ? B64 : A64;
         V* d = (kk & 1) ? B : A;
-        launch_stage<double2>(st, adj, c64, b, 1, d64, b, 1, b, s);
+        reference([&] { launch_stage<double2>(st, adj, c64, b, 1, d64, b, 1, b, s); });
         launch_stage<V>(st, adj, c, b, 1, d, b, 1, b, s);
         record(d64, d, (adj ? st.in_len : st.out_len) * (long long)b);
         c64 = d64;
@@ -1839,7 +1874,7 @@ int stage_errors_t(fio_op op, int which, const void* x, int64_t ld, int b, cudaS
     if (which >= 2) {
       const int h0 = op->n_bf, nh = op->n_hif;
       auto step = [&](const Stage& st, bool adj) {
-        inplace_stage<double2>(st, adj, W64, A64, b, b, s);
+        reference([&] { inplace_stage<double2>(st, adj, W64, A64, b, b, s); });
         inplace_stage<V>(st, adj, W, A, b, b, s, B, op->max_len);
         record(W64, W, N * b);
       };
@@ -1875,7 +1910,10 @@ extern "C" int fio_stage_errors(fio_op op, int which, const void* x, int64_t ld,
   if (which >= 2 && op->n_root == 0) return FIO_ENOTSUP;
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaGetLastError() != cudaSuccess) return FIO_ECUDA;
-  if (precision == FIO_PDF && df_as_fp64(op, b)) return stage_errors_t<double2>(op, which, x, ld, b, s, errs, cap, nerr);
+  if (precision == FIO_PDF && df_as_fp64(op, b)) {
+    ForDf in_fp64(true);
+    return stage_errors_t<double2>(op, which, x, ld, b, s, errs, cap, nerr);
+  }
   if (precision == FIO_PDF) return stage_errors_t<dfc>(op, which, x, ld, b, s, errs, cap, nerr);
   TcMode m(tc_mode_of(precision));
   return stage_errors_t<float2>(op, which, x, ld, b, s, errs, cap, nerr);

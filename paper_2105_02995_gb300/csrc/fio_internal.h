@@ -50,10 +50,10 @@ struct Stage {
   const int2* t128_adj = nullptr;
   int n128_fwd = 0, n128_adj = 0;
   // kernel variant chosen by fio_autotune per [arithmetic: c128, c64, double-float, TF32, BF16,
-  // split TF32][direction: forward, adjoint][right-hand-side bucket]; 0 = the built-in choice
-  // (see fio_capi.cu)
+  // split TF32, c128 on behalf of FIO_PDF][direction: forward, adjoint][right-hand-side bucket]; 0 = the
+  // built-in choice (see fio_capi.cu)
   bool x3_pinned[5] = {};  // per bucket: the split-TF32 variant was set by fio_set_variant, not by the autotuner
-  int8_t var[6][2][5] = {};
+  int8_t var[7][2][5] = {};
   // TMA tensor maps of the tensor-core A operands per [direction: forward (M32 / Mbf), adjoint
   // (M32t / Mbft)][element: FP32, BF16]; tma_ok marks the maps that encoded (16-byte aligned
   // rows and base)
