@@ -855,24 +855,20 @@ bool launch_tc_var(const TcArgs& a, int ncta, cudaStream_t s, int var) {
   }
 }
 
-// multiprocessor count of the current device (cached per device)
+// multiprocessor count of the current device (cached per thread for the last device: every stage launch asks)
 int num_sms() {
-  static std::mutex mu;
-  static std::map<int, int> cache;
+  thread_local int last = -1, n = 1;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
-  std::lock_guard<std::mutex> lock(mu);
-  auto it = cache.find(dev);
-  if (it != cache.end()) return it->second;
-  int n = 0;
+  if (dev == last) return n;
   if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
     cudaGetLastError();
     n = 1;
   }
-  cache[dev] = n;
+  last = dev;
   return n;
 }
 

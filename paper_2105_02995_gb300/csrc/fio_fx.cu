@@ -58,14 +58,12 @@ bool opt_in(const void* f, int bytes) {
 }
 
 int sm_count() {
-  static std::mutex mu;
-  static std::map<int, int> known;
-  int dev = 0, n = 0;
+  thread_local int last = -1, n = 1;
+  int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  std::lock_guard<std::mutex> lock(mu);
-  int& k = known[dev];
-  if (k == 0) k = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 1;
-  return k;
+  if (dev != last && (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)) n = 1;
+  last = dev;
+  return n;
 }
 
 template <typename R, bool ADJ, int BT>
