@@ -473,9 +473,16 @@ int fio_scratch(fio_op op, int b, size_t elem, cudaStream_t s, void** bufs, void
   }
   if (rc) return rc;
   for (int k = 0; k < 5; ++k) bufs[k] = (uint8_t*)op->scratch + k * per_al;
-  // no room for the fixed-point kernel's: this call runs on the CUDA cores
+  // no room for the fixed-point kernel's: this call runs on the CUDA cores (so does a captured call whose
+  // sizing call had none: nothing may be allocated now)
   const size_t fxneed = fxbuf ? fx_scratch_bytes(op, b, elem) : 0;
-  rc = fxneed ? grow(&op->fx_scratch, &op->fx_scratch_bytes, fxneed) : FIO_ENOMEM;
+  auto captured = [&] {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const bool yes = cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+    if (yes) cudaGetLastError();
+    return yes;
+  };
+  rc = fxneed && (fxneed <= op->fx_scratch_bytes || !captured()) ? grow(&op->fx_scratch, &op->fx_scratch_bytes, fxneed) : FIO_ENOMEM;
   if (rc == FIO_ECUDA) return rc;
   if (fxbuf) *fxbuf = rc == FIO_OK ? op->fx_scratch : nullptr;
   if (fxbytes) *fxbytes = rc == FIO_OK ? fxneed : 0;
@@ -1071,9 +1078,10 @@ template <typename V>
 bool fx_rule(const Stage& st, bool adj, int b, bool pinned) {
   constexpr bool W = std::is_same<V, double2>::value;
   if (std::is_same<V, dfc>::value || !g_fx_scratch || (!W && g_tc_mode != 0 && !g_fx_corrections)) return false;
-  // FP32 by the built-in rule in the solvers' split-TF32 corrections only: 30 bits below a row's and a
-  // column's largest are too few for the butterfly factors of a real operator (generalized Radon transform
-  // n = 256, b = 32, against the FP64 apply: 1.4e-6 on the CUDA cores, 7.7e-6 so, 2.4e-5 in split TF32)
+  // FP32 by the built-in rule in the solvers' split-TF32 corrections only.  Taken back for FP32 applies when
+  // the factor's rows alone were scaled: 7.7e-6 off the FP64 apply on a real operator (generalized Radon
+  // transform n = 256), lost in the HIF stages, against 1.4e-6 on the CUDA cores.  With column scales
+  // 9.3e-7 (K-dot 1.9e-7 against 1.2e-6, G-dot 8.8e-7 against 7.3e-7; split TF32 3.2e-5)
   if (!W && !pinned && !g_fx_corrections) return false;
   return st.fx_ok[W ? 0 : 1] && (pinned || fx_takes(st, adj, W, b));
 }

@@ -98,11 +98,19 @@ def test_scratch_that_does_not_fit_is_asked_for_again(packed):
     op.set_variant(wide, binding.FIO_P64, 0)
     op.release()
     op = binding.Operator(packed)
+    torch.cuda.Stream()  # torch's streams are made before memory is short
     pool = 5 * 16 * N * wide  # and 1/5 of it for the fixed-point kernel
     with Hog(pool + pool // 10):
         op.apply_K(x, out)
         torch.cuda.synchronize()
         assert held(op) >= pool
+        assert torch.equal(out, cores)
+        graph = torch.cuda.CUDAGraph()  # a captured call allocates nothing either
+        with torch.cuda.graph(graph):
+            op.apply_K(x, out)
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
     assert torch.equal(out, cores)
     assert torch.equal(op.apply_K(x8), want8)
     assert not torch.equal(op.apply_K(x, out), cores)
