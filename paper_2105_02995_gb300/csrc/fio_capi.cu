@@ -538,7 +538,11 @@ int num_sms();
 //     double-float               0.93           1.03 (30000)   Example 3 n = 32, b = 16
 //     FP64  40 tiles 64 x 230    0.46           1.05 (8000)    PCG, b = 5
 //   more                         110000         smaller
-//     FP32  1D N = 16384 b = 16  0.94           1.05 (30000)
+//     FP32  1D N = 16384 b = 16  0.94           1.03 (80000)   K-dot*; inverse 1.38 and 1.49
+//           1D N = 4096 b = 16   0.92           1.22 (80000, 1.10 at 34000)
+//           2D n = 128 b = 6     0.74           1.08 (80000)   K-dot*; inverse 0.92 and 1.11
+//           1D N = 65536 b = 16  1.41           1.29 (80000)   inverse; 7 times as many CTAs as SMs: from
+//           four on the waves even themselves out
 //     FP64  1D N = 4096 b = 1    0.65           1.18 (2500, 0.65 at 8000)   K-dot*
 constexpr long long kLightMacs = 110000;
 template <bool ADJ, typename V>
@@ -546,7 +550,7 @@ bool light(const StageArgs<V>& a, int rows, int rhs, const dim3& grid) {
   const long long ctas = (long long)grid.x * grid.y * grid.z, sms = num_sms();
   const bool many = 2 * ctas > sms;
   const long long limit = 8 * ctas <= sms                    ? kLightMacs
-                          : sizeof(V) == sizeof(float2)      ? (many ? 34000 : kLightMacs)
+                          : sizeof(V) == sizeof(float2)      ? (many && ctas <= 4 * sms ? 80000 : kLightMacs)
                           : std::is_same<V, dfc>::value      ? (many ? 30000 : 50000)
                                                              : (many ? 2500 : 12000);
   return (long long)rows * (ADJ ? a.R : a.C) * std::min(rhs, a.b) <= limit * a.ksplit;
