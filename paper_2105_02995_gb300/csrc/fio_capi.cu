@@ -1641,15 +1641,16 @@ int tune_type(fio_op op, int b, cudaStream_t s, int* choices, int cap, int* nch)
       const bool tc = use_tc<V>(st, b, adj);
       const int ti = tc ? 2 + g_tc_mode : var_table<V>();
       int best = 0;
-      if (g_for_df && fx_takes(st, adj, true, b)) {
-        best = kFxVariant;  // what FIO_PDF runs in FP64 for: several times as fast as the CUDA-core tiles
-      } else if (st.nblk > 0) {
+      // FIO_PDF runs in FP64 for the fixed-point kernel, several times as fast as the CUDA-core tiles where its rule
+      // takes the stage: against it only the warp kernel is timed there (16-point leaf stages at wide batches)
+      const bool fx_or_small = g_for_df && fx_takes(st, adj, true, b);
+      if (st.nblk > 0) {
         const StageArgs<V> a = stage_args<V>(st, adj, X, rs, 1, Y, rs, 1, b);
         float tbest = -1.f;
         const int ncand = tc ? 9 : kNCand + 1;
         for (int k = 0; k < ncand; ++k) {
           const int var = tc ? kTcCand[k] : (k == kNCand ? kFxVariant : kCand[bucket][k]);
-          if (var <= 0 && !tc) continue;
+          if ((var <= 0 && !tc) || (fx_or_small && var != kFxVariant && var != kSmallVariant)) continue;
           if (var == kFxVariant && (ti == 1 || !fx_rule<V>(st, adj, b, true))) continue;
           float t;
           if (st.kind == 1) {
