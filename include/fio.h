@@ -29,8 +29,10 @@
  * per step, FP32 accumulation; the dropped tail*tail term is ~2^-22 relative); same factors and
  * vectors as FIO_PTF32.  With fewer than 8 right-hand sides the tensor-core precisions fall back
  * to the FP32 CUDA-core kernels.  The large stages of FIO_P64 (and of FIO_P32 under variant 50) run on the tensor cores in
- * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below their row's and column's largest,
- * digit products summed exactly, each output rounded once (columns with infinities, NaN or extreme exponents are summed plainly).  The
+ * fixed point: operands cut to 62 (FP64) or 30 (FP32) bits below the largest of a block's scaled row and of
+ * its gathered column, digit products summed exactly, each output rounded once.  An output's error is a bound
+ * on the block's largest scaled product, not on its own sum as an FMA chain's is: outputs far below the
+ * others of their block keep fewer digits.  (Columns with infinities, NaN or extreme exponents are summed plainly.)  The
  * digit copies that this takes (FP32's with FIO_MASK_TC only) are made at upload where they fit half of the
  * free device memory, FP64's first.
  * fio_solve's corrections with inner = FIO_PTF32X3 take them too (see there).
@@ -259,7 +261,9 @@ int fio_stage_errors(fio_op op, int which, const void* x, int64_t ld, int b, int
 int fio_query(fio_op op, int* d, int64_t* n, int64_t* N, size_t* device_bytes);
 
 /* Stage counts and the number of kernel launches one apply issues (for launch accounting):
- * which = 0 apply_K, 1 apply_Kadj, 2 apply_G, 3 apply_inv. */
+ * which = 0 apply_K, 1 apply_Kadj, 2 apply_G, 3 apply_inv.  Counted as the CUDA-core and tensor-core kernels
+ * of the complex64 precisions run: a stage in fixed point (FIO_P64, FIO_PDF) is two launches, a gather and the
+ * product, and has no copy-back. */
 int fio_launch_count(fio_op op, int which, int b, int* launches);
 
 /* Diagnostics: the apply `which` (as in fio_launch_count) with a CUDA event recorded on `stream`
