@@ -80,9 +80,11 @@ bool launch(FxArgs a, uint8_t* X, int* ej, cudaStream_t s) {
   // 1D N = 16384 b = 5, 15 K steps: 414 us without, 360 with)
   const bool early = (long long)a.steps * a.nrt <= 300LL * sm_count();
   const int groups = (a.maxcols + 4 * (256 / BT) - 1) / (4 * (256 / BT));
+  // (four groups kept take 126 registers: where the CTAs are more than two a multiprocessor, the loop of 54
+  // is no slower; 2D n = 256 FP64 b = 1, K-dot 2031 us with four, 2023 without)
   auto gather = groups <= 1   ? k_fx_gather<R, ADJ, BT, 1>
                 : groups <= 2 ? k_fx_gather<R, ADJ, BT, 2>
-                : groups <= 4 ? k_fx_gather<R, ADJ, BT, 4>
+                : groups <= 4 && (long long)a.nblk * a.nrt <= 2LL * sm_count() ? k_fx_gather<R, ADJ, BT, 4>
                               : k_fx_gather<R, ADJ, BT, 0>;
   pdl_launch(early, gather, dim3((unsigned)a.nblk, (unsigned)a.nrt), 256, 0, s, a, X, ej);
   pdl_launch(true, k_stage_fx<R, ADJ, BT>, (unsigned)std::min<long long>(total, sm_count()), fx::kThreads, need, s, a);

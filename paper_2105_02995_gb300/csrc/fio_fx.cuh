@@ -55,8 +55,8 @@
 // it from one another.  Registers are moved to the drain warps (setmaxnreg), which keep a row's sums.
 //
 // Measured (one GB300, the shapes of the 2D transform at n = 256, 548 M entries, K-dot; before: the
-// best CUDA-core kernel): FP64 b = 1 / 8 / 16 / 32: 5.53 / 32.9 / 65.6 / 129 ms before, 2.03 / 2.26 /
-// 3.07 / 5.96 now; FP32 b = 16 / 32: 2.26 / 3.45 before, 1.53 / 1.94 now.  On 64 blocks of 512 x 512, FP64 b = 16, a K step
+// best CUDA-core kernel): FP64 b = 1 / 8 / 16 / 32: 5.53 / 32.9 / 65.6 / 129 ms before, 2.02 / 2.25 /
+// 3.07 / 5.97 now; FP32 b = 16 / 32: 2.26 / 3.45 before, 1.53 / 1.94 now.  On 64 blocks of 512 x 512, FP64 b = 16, a K step
 // takes 0.65 us (1340 clocks); it moves 147 KB through shared memory (copies in 18, read 18, digits
 // written 40, operands read 71), 1150 clocks at 128 bytes a clock: L1 and shared memory are 73% busy on the busiest
 // SM, the tensor cores 46%, HBM 43% (its stream needs 760 clocks).
