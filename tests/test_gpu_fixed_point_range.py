@@ -25,18 +25,18 @@ def gaussian(rng, *shape):
     return rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
 
 
-def operator(kind, map_block, hif_block):
+def operator(kind, map_block, hif_block, sides=SIDES):
     """Three butterfly stages and a HIF level of ragged blocks above 4096 unknowns, where every FP64
     stage takes the kernel from five right-hand sides on."""
     if kind not in _ops:
         fbuild.build()
         rng = np.random.default_rng(7)
-        N = sum(SIDES)
+        N = sum(sides)
 
         def stage(inplace):
             st, i = Stage(KIND_INPLACE if inplace else KIND_MAP, N, N), 0
             pin, pout = rng.permutation(N), rng.permutation(N)
-            for m in rng.permutation(SIDES):
+            for m in rng.permutation(sides):
                 rows = pin if inplace else pout
                 st.add((hif_block if inplace else map_block)(rng, m), pin[i:i + m], rows[i:i + m])
                 i += m
@@ -121,3 +121,21 @@ def test_error_no_larger_than_an_fma_chain(kind, vector):
         assert not np.array_equal(y, z)  # the two kernels
         ey, ez = (float(np.sqrt((np.abs(v - want) ** 2).sum() / (np.abs(want) ** 2).sum())) for v in (y, z))
         assert ey <= ez, (w, ey, ez)
+
+
+@pytest.mark.parametrize("b", [1, 8, 9, 16, 17, 32, 33])
+@pytest.mark.parametrize("prec", [binding.FIO_P64, binding.FIO_P32])
+def test_short_blocks(prec, b):
+    """Stages whose gathers keep all of a thread's entries (blocks of at most 58 columns), some of one column.
+    FP32: 2 2^-24 a stage, as in test_gpu_fixed_point."""
+    op, P, N = operator("short", even, near_identity, [1, 2, 33, 57] + [58] * 110)
+    wide = prec == binding.FIO_P64
+    xd = dev(gaussian(np.random.default_rng(b), N, b), torch.complex128 if wide else torch.complex64)
+    x = xd.cpu().numpy().astype(np.complex128)
+    try:
+        op.set_variant(b, prec, 50)
+        for w in ("K", "Kadj"):
+            y = getattr(op, "apply_" + w)(xd, precision=prec).cpu().numpy().astype(np.complex128)
+            assert rel(y, REFS[w](P, x)) < (TOL64 if wide else 1.1e-6), w
+    finally:
+        op.set_variant(b, prec, 0)
