@@ -111,7 +111,9 @@ __global__ void k_basis_sub(const double2* V, long long vstride, double2* w, lon
 }
 
 // y[:, j] = alpha[j] x[:, j] + beta[j] y[:, j]   (x, y with leading dimensions), the scalars of up to
-// kCoefs columns as launch parameters: no copy, and nothing for the host to wait for
+// kCoefs columns as launch parameters: no copy, and nothing for the host to wait for.  With beta = 0 y is
+// not read: the first search direction and the basis vectors are written into memory that nothing has set, and 0 times
+// what happens to lie there may be NaN
 constexpr int kCoefs = 96;
 struct Coefs {
   double2 a[kCoefs], b[kCoefs];
@@ -125,7 +127,7 @@ __global__ void k_axpby(const __grid_constant__ Coefs q, const double2* x, long 
   const int j = (int)(t / N);
   const long long i = t - (long long)j * N;
   const double2 a = q.a[j], bb = q.b[j];
-  const double2 xv = x[i + j * ldx], yv = y[i + j * ldy];
+  const double2 xv = x[i + j * ldx], yv = bb.x == 0.0 && bb.y == 0.0 ? make_double2(0.0, 0.0) : y[i + j * ldy];
   double2 r;
   r.x = a.x * xv.x - a.y * xv.y + bb.x * yv.x - bb.y * yv.y;
   r.y = a.x * xv.y + a.y * xv.x + bb.x * yv.y + bb.y * yv.x;
